@@ -12,6 +12,7 @@
 //   q^{n+1} = q^n + sum_i (b_i dtM^{-1}NL_i + b~_i dtM^{-1}L_i)                          (combine)
 // The identity M^{-1} L_i = (Q - R1)/(dt a~_ii) holds exactly for the recovered Q because
 // the local rows of the stage system are solved exactly (eq. IMEXRKDiscretizedForm).
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -25,6 +26,7 @@
 
 #include "hdgdg.h"
 #include "internal.h"
+#include "solve.h"
 
 using namespace hdgdg;
 
@@ -70,6 +72,12 @@ bool explicit_scheme(const hdgdg_config* c) { return c->scheme == HDGDG_RK2 || c
 
 int restart_of(const hdgdg_config* c) { return c->krylov_restart > 0 ? c->krylov_restart : 10; }
 
+// Krylov basis vectors in global memory (at least what the one-launch solve keeps there instead)
+size_t basis_vectors(const hdgdg_config* c) {
+    const int m1 = restart_of(c) + 1;
+    return (size_t)(matrix_free(c) ? m1 : std::max(m1, solve_basis_vectors(c->precision == HDGDG_MIXED)));
+}
+
 // order of the trace-solve initial guess (0: start from zero)
 int guess_order(const hdgdg_config* c) { return c->krylov_guess < 0 ? 0 : c->krylov_guess == 0 ? 5 : c->krylov_guess; }
 
@@ -110,12 +118,13 @@ Plan make_plan(const hdgdg_config* c) {
     b += 5 * p.nt * d;                                        // g, x~, qhat, w, DG face fluxes
     if (c->precision == HDGDG_MIXED) {                        // FP32 S~, FP32 basis and work vector
         if (!matrix_free(c)) b += n_edges * 6 * (size_t)p.NF * p.NF * sizeof(float);
-        b += ((size_t)p.m + (matrix_free(c) ? 4 : 2)) * p.nt * sizeof(float);   // basis and w (three, matrix-free)
+        b += (basis_vectors(c) + (matrix_free(c) ? 3 : 1)) * p.nt * sizeof(float);   // basis and w (three, matrix-free)
     } else {
-        b += ((size_t)p.m + 1) * p.nt * d;                    // FP64 Krylov basis
+        b += basis_vectors(c) * p.nt * d;                     // FP64 Krylov basis
     }
     b += (reduction_scratch_doubles(p.m, (int)n_edges, (int)P) + mass_scratch_doubles() + 4 * (size_t)(p.m + 2) + 16) * d;
     b += 64 + sizeof(GmresCtl);                               // flags, GMRES control block
+    if (!matrix_free(c)) b += solve_part_bytes(kSolveMaxBlocks) + 128;  // the one-launch solve's exchanges
     if (c->local_precision == HDGDG_LOCAL_FP32) b += n_el * (size_t)p.NV * p.NV * sizeof(float);
     if (c->local_precision == HDGDG_LOCAL_BF16) b += tc_image_bytes((int)P);
     if (c->local_precision == HDGDG_LOCAL_BF16_SPLIT) b += tc_split_image_bytes((int)P);
@@ -347,6 +356,10 @@ struct hdgdg_sim {
     double *red = nullptr, *mred = nullptr, *dvals = nullptr;
     GmresCtl* ctl = nullptr;
     CycleGraph cycle_graph[4];   // [FP64 form, mixed form] x [timers off, on]
+    // the trace solve as one cooperative launch (small and mid-size systems on the assembled matrix)
+    SolvePlan splan;
+    unsigned long long* solve_part = nullptr;
+    unsigned* solve_epoch = nullptr;   // then the count, and at 16 words the launch's SolveClocks
     std::vector<StepGraph> step_graphs;   // whole-step graphs (host_steps = 0, timers off)
     SolveCtl* sctl = nullptr;             // device-side control of the solve being replayed
     DevHist* dhist = nullptr;             // each stage's guess history, as the step graph reads it
@@ -647,9 +660,14 @@ cudaError_t cycle_enqueue(hdgdg_sim* sim, const double* g, cudaStream_t st, bool
 // T = double: the FP64 form.  T = float (mixed form): the cycle runs on the FP32 copy of S~
 // and FP32 basis vectors; every cycle starts from the true residual r = g - S~ x~ computed in
 // FP64 and adds its correction to the FP64 x~ (iterative refinement).
+void rotate_history(hdgdg_sim* sim, int stage);
+template <typename T>
+hdgdg_status solve_one_launch(hdgdg_sim* sim, const double* g, double* qhat, int* iters, double* relres, int stage);
+
 template <typename T>
 hdgdg_status gmres_solve(hdgdg_sim* sim, const double* g, double* qhat, int* iters, double* relres,
                          int stage) {
+    if (sim->splan.on) return solve_one_launch<T>(sim, g, qhat, iters, relres, stage);
     constexpr bool kMixed = sizeof(T) == sizeof(float);
     const size_t n = sim->plan.nt;
     const double rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
@@ -825,21 +843,14 @@ hdgdg_status gmres_solve(hdgdg_sim* sim, const double* g, double* qhat, int* ite
     const int order = guess_order(&sim->cfg);
     if (stage >= 0 && order > 0) {   // keep x~ and S~ x~ = g - r for the next steps' guesses
         TimedGroup tg(sim, HDGDG_KT_GUESS);
-        double* ox = sim->xhist[stage][order - 1];
-        double* oy = sim->yhist[stage][order - 1];
-        for (int j = order - 1; j > 0; --j) {
-            sim->xhist[stage][j] = sim->xhist[stage][j - 1];
-            sim->yhist[stage][j] = sim->yhist[stage][j - 1];
-        }
-        sim->xhist[stage][0] = ox;
-        sim->yhist[stage][0] = oy;
-        CU(cudaMemcpyAsync(ox, sim->xt, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+        rotate_history(sim, stage);
+        double* oy = sim->yhist[stage][0];
+        CU(cudaMemcpyAsync(sim->xhist[stage][0], sim->xt, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
         CombineTerms r{};   // sim->w holds the final true residual g - S~ x~
         r.n = 1;
         r.X[0] = sim->w;
         r.c[0] = -1.0;
         CU(launch_combine(n, g, r, oy, nullptr, st));
-        sim->n_hist[stage] = std::min(sim->n_hist[stage] + 1, order);
     }
     *iters = total;
     *relres = rnorm / bnorm;
@@ -898,6 +909,115 @@ cudaError_t dg_nl_enqueue(hdgdg_sim* sim, const double* Qi, bool stage_value, do
     return launch_dg_nl(sim->g, Qi, sim->phiB, sim->tau, sim->cfg.dt, sim->fface, out, st, t);
 }
 
+// ---- the trace solve as one launch ----------------------------------------------------------------
+// The whole solve of gmres_solve -- start, restart cycles, back-transformation, history store --
+// enqueued on st as one cooperative launch (kernels_solve.inl); its counters are added to sstats.
+// dh: the stage's history table (nullptr: none).  The least-squares start keeps its own kernels, and
+// the launch takes over from the start they chose.
+template <typename T>
+cudaError_t solve_enqueue_one_launch(hdgdg_sim* sim, const double* g, double* qhat, const DevHist* dh,
+                                     SolveClocks* clocks, cudaStream_t st) {
+    constexpr bool kMixed = sizeof(T) == sizeof(float);
+    const size_t n = sim->plan.nt;
+    SolveArgs a{};
+    a.plan = sim->splan;
+    a.n_edges = sim->g.n_edges;
+    a.m = sim->plan.m;
+    a.twice = !kMixed || sim->cfg.krylov_ortho != 1;
+    a.S64 = sim->Stil;
+    a.St = kMixed ? static_cast<const void*>(sim->Stil32) : sim->Stil;
+    a.Slo = sim->Stil_lo;
+    a.col = sim->Scol;
+    a.Minv = sim->Minv;
+    a.minv_pairs = sim->minv_pairs;
+    a.g = g;
+    a.xt = sim->xt;
+    a.w = sim->w;
+    a.qhat = qhat;
+    // the global basis' bytes hold what crosses blocks
+    a.A = kMixed ? reinterpret_cast<unsigned long long*>(sim->V32) : reinterpret_cast<unsigned long long*>(sim->V);
+    a.X = a.A + (kMixed ? 2 : 4) * n;
+    a.part = sim->solve_part;
+    a.epoch = sim->solve_epoch;
+    a.count = sim->solve_epoch + 1;
+    a.error = spmv_error(sim);
+    a.dh = dh;
+    std::memcpy(a.coef, kGuessCoef, sizeof(kGuessCoef));
+    a.rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
+    a.maxit = sim->cfg.krylov_maxit > 0 ? sim->cfg.krylov_maxit : 2000;
+    a.stagnation = kStagnationFloor;
+    a.sc = sim->sctl;
+    a.ss = sim->sstats;
+    a.clocks = clocks;
+    if (kMixed && dh && sim->cfg.krylov_guess_ls) {
+        cudaError_t e = launch_multidot(g, 0, 1, g, n, sim->red, sim->dls + 32, st, &dh->has_history);
+        if (e == cudaSuccess) e = launch_guess_gram_dev(n, g, dh, sim->red, sim->dls, st);
+        if (e == cudaSuccess)
+            e = launch_ls_start_dev(n, g, dh, sim->dls, a.rtol, 1e-6, a.maxit, sim->ctl, sim->sctl, sim->sstats,
+                                    dv_nrm(sim), sim->xt, sim->w, st);
+        if (e != cudaSuccess) return e;
+        a.start_given = true;
+    }
+    return kMixed ? launch_solve_f32(sim->g.P, a, st) : launch_solve_f64(sim->g.P, a, st);
+}
+
+cudaError_t upload_history(hdgdg_sim* sim, cudaStream_t st);
+
+// gmres_solve on a handle whose solves are one launch: the host waits once, for the result.
+template <typename T>
+hdgdg_status solve_one_launch(hdgdg_sim* sim, const double* g, double* qhat, int* iters, double* relres, int stage) {
+    cudaStream_t st = sim->stream;
+    const bool history = stage >= 0 && guess_order(&sim->cfg) > 0;
+    CU(cudaMemsetAsync(sim->sstats, 0, sizeof(StepStats), st));
+    if (history) CU(upload_history(sim, st));
+    cudaEvent_t ea = sim->timing ? take_event(sim) : nullptr, eb = ea ? take_event(sim) : nullptr;
+    SolveClocks* clocks = eb ? reinterpret_cast<SolveClocks*>(sim->solve_epoch + 16) : nullptr;
+    if (eb) CU(cudaEventRecord(ea, st));
+    CU(solve_enqueue_one_launch<T>(sim, g, qhat, history ? sim->dhist + stage : nullptr, clocks, st));
+    if (eb) CU(cudaEventRecord(eb, st));
+    CU(cudaMemcpyAsync(sim->hbuf, sim->flags, 4 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    CU(cudaMemcpyAsync(sim->hbuf + 4, sim->sstats, sizeof(StepStats), cudaMemcpyDeviceToHost, st));
+    if (clocks) CU(cudaMemcpyAsync(sim->hbuf + 16, clocks, sizeof(SolveClocks), cudaMemcpyDeviceToHost, st));
+    TRY(sync(sim));
+    unsigned flag[4];
+    StepStats ss;
+    std::memcpy(flag, sim->hbuf, sizeof(flag));
+    std::memcpy(&ss, sim->hbuf + 4, sizeof(ss));
+    if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
+    if (eb) {   // the launch's time, divided among the kernel classes as its first block's clock saw them
+        SolveClocks ck;
+        std::memcpy(&ck, sim->hbuf + 16, sizeof(ck));
+        const long long part[5] = {ck.spmv, ck.ortho, ck.residual, ck.guess, ck.precond};
+        const int cls[5] = {HDGDG_KT_SPMV, HDGDG_KT_ORTHO, HDGDG_KT_RESIDUAL, HDGDG_KT_GUESS, HDGDG_KT_PRECOND};
+        const long long count[5] = {ss.its, ss.its, ss.cycles, 1, 1};
+        long long total = 0;
+        for (long long v : part) total += v;
+        float ms = 0.f;
+        if (total > 0 && cudaEventElapsedTime(&ms, ea, eb) == cudaSuccess) {
+            for (int i = 0; i < 5; ++i) {
+                sim->kt_ms[cls[i]] += ms * ((double)part[i] / (double)total);
+                sim->kt_n[cls[i]] += count[i];
+            }
+        } else {
+            cudaGetLastError();
+        }
+    }
+    if (ea) sim->ev_pool.push_back(ea);
+    if (eb) sim->ev_pool.push_back(eb);
+    *iters = ss.last_its;
+    *relres = ss.last_rel;
+    sim->stats.last_krylov_iterations = ss.last_its;
+    sim->stats.last_rel_residual = ss.last_rel;
+    if (ss.nonfinite) return fail(sim, HDGDG_ENONFINITE, "non-finite trace right-hand side or GMRES residual");
+    sim->stats.last_guess_order = ss.last_guess;
+    if (ss.notconv)
+        return fail(sim, HDGDG_ENOTCONVERGED, "GMRES: relative residual %.3e above the tolerance after %d iterations",
+                    ss.notconv_rel, ss.notconv_its);
+    sim->stats.krylov_iterations += ss.its;
+    if (history) rotate_history(sim, stage);
+    return HDGDG_OK;
+}
+
 // ---- whole-step graphs ------------------------------------------------------------------------
 // The trace solve of gmres_solve with every host decision moved to the device (kernels_ctl.cu),
 // enqueued on st while a whole time step is being captured: the candidate norms, the choice of the
@@ -915,6 +1035,7 @@ cudaError_t solve_enqueue_graph(hdgdg_sim* sim, const double* g, double* qhat, i
     const double inner_rel = kMixed ? 1e-6 : 0.0;
     const int order = guess_order(&sim->cfg);
     const bool history = stage >= 0 && order > 0;
+    if (sim->splan.on) return solve_enqueue_one_launch<T>(sim, g, qhat, history ? sim->dhist + stage : nullptr, nullptr, st);
     cudaError_t e = cudaSuccess;
     if (history && kMixed && sim->cfg.krylov_guess_ls) {   // the least-squares start, from the device table
         const DevHist* dh = sim->dhist + stage;
@@ -1012,7 +1133,8 @@ cudaError_t step_enqueue_graph(hdgdg_sim* sim, cudaStream_t st, StepGraph& sg) {
                             sim->Qs32 && sim->cfg.dg_precision != 1 && sim->At[sim->s - 1][sim->s - 1] != 0.0;
     // each stage's history store reads x~, g and r, which nothing overwrites before the next
     // stage's condensation: it runs on a branch beside the recovery and the DG residual
-    const bool branch = !sim->ens && sim->side_stream && guess_order(&sim->cfg) > 0;
+    // (the one-launch solve stores it itself)
+    const bool branch = !sim->ens && !sim->splan.on && sim->side_stream && guess_order(&sim->cfg) > 0;
     int pending = -1;   // the stage whose store has not joined yet
     for (int i = 0; i < sim->s && e == cudaSuccess; ++i) {
         const double* Qi = sim->q;
@@ -1101,6 +1223,20 @@ cudaError_t upload_history(hdgdg_sim* sim, cudaStream_t st) {
     return cudaMemcpyAsync(sim->dhist, sim->hhist, sim->s * sizeof(DevHist), cudaMemcpyHostToDevice, st);
 }
 
+// The slot a solve of this stage wrote last becomes its newest.
+void rotate_history(hdgdg_sim* sim, int i) {
+    const int order = guess_order(&sim->cfg);
+    double* ox = sim->xhist[i][order - 1];
+    double* oy = sim->yhist[i][order - 1];
+    for (int j = order - 1; j > 0; --j) {
+        sim->xhist[i][j] = sim->xhist[i][j - 1];
+        sim->yhist[i][j] = sim->yhist[i][j - 1];
+    }
+    sim->xhist[i][0] = ox;
+    sim->yhist[i][0] = oy;
+    sim->n_hist[i] = std::min(sim->n_hist[i] + 1, order);
+}
+
 void drop_step_graphs(hdgdg_sim* sim) {
     for (auto& sg : sim->step_graphs)
         if (sg.exec) cudaGraphExecDestroy(sg.exec);
@@ -1161,7 +1297,7 @@ hdgdg_status one_step_graph(hdgdg_sim* sim) {
     if (bad) {   // the history slots may hold this step's partial solves: start the next solves afresh
         for (int i = 0; i < sim->s; ++i) sim->n_hist[i] = 0;
         if (flag[2]) return fail(sim, HDGDG_ECUDA, "a bounded wait of a local kernel ran out (%u)", flag[2]);
-        if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the pipelined SpMV ran out (%u)", flag[3]);
+        if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
         if (ss.nonfinite) return fail(sim, HDGDG_ENONFINITE, "non-finite trace right-hand side or GMRES residual");
         if (ss.notconv) {
             sim->stats.last_krylov_iterations = ss.notconv_its;
@@ -1171,19 +1307,8 @@ hdgdg_status one_step_graph(hdgdg_sim* sim) {
         }
         return fail(sim, HDGDG_ENONFINITE, "step %lld produced a non-finite state", sim->stats.steps + 1);
     }
-    const int order = guess_order(&sim->cfg);
-    for (int i = 0; i < sim->s && order > 0; ++i) {   // the slot written last becomes the newest
-        if (sim->At[i][i] == 0.0) continue;
-        double* ox = sim->xhist[i][order - 1];
-        double* oy = sim->yhist[i][order - 1];
-        for (int j = order - 1; j > 0; --j) {
-            sim->xhist[i][j] = sim->xhist[i][j - 1];
-            sim->yhist[i][j] = sim->yhist[i][j - 1];
-        }
-        sim->xhist[i][0] = ox;
-        sim->yhist[i][0] = oy;
-        sim->n_hist[i] = std::min(sim->n_hist[i] + 1, order);
-    }
+    for (int i = 0; i < sim->s && guess_order(&sim->cfg) > 0; ++i)
+        if (sim->At[i][i] != 0.0) rotate_history(sim, i);
     std::swap(sim->q, sim->q_new);
     sim->stats.steps += 1;
     sim->t += sim->cfg.dt;
@@ -1283,7 +1408,7 @@ hdgdg_status one_step(hdgdg_sim* sim) {
     TRY(sync(sim));
     std::memcpy(flag, &sim->hbuf[0], sizeof(flag));
     if (flag[2]) return fail(sim, HDGDG_ECUDA, "a bounded wait of a local kernel ran out (%u)", flag[2]);
-    if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the pipelined SpMV ran out (%u)", flag[3]);
+    if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
     if (flag[0]) return fail(sim, HDGDG_ENONFINITE, "step %lld produced a non-finite state", sim->stats.steps + 1);
     std::swap(sim->q, sim->q_new);
     sim->stats.steps += 1;
@@ -1366,10 +1491,10 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
             TRY(dalloc(sim, &sim->Stil32, (size_t)g.n_edges * 6 * p.NF * p.NF));
             if (c->residual_f32x2) TRY(dalloc(sim, &sim->Stil_lo, (size_t)g.n_edges * 6 * p.NF * p.NF));
         }
-        TRY(dalloc(sim, &sim->V32, (size_t)(p.m + 1) * p.nt));
+        TRY(dalloc(sim, &sim->V32, basis_vectors(c) * p.nt));
         TRY(dalloc(sim, &sim->w32, (matrix_free(c) ? 3 : 1) * p.nt));   // matrix-free: w1 and two alternating outputs
     } else {
-        TRY(dalloc(sim, &sim->V, (size_t)(p.m + 1) * p.nt));
+        TRY(dalloc(sim, &sim->V, basis_vectors(c) * p.nt));
     }
     TRY(dalloc(sim, &sim->red, reduction_scratch_doubles(p.m, g.n_edges, g.P)));
     CU(cudaMemset(sim->red, 0, sizeof(double)));   // the reductions' ticket counter starts at zero
@@ -1382,6 +1507,17 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
     TRY(dalloc(sim, &sim->dhist, kMaxStages));
     CU(cudaMallocHost(&sim->hhist, kMaxStages * sizeof(DevHist)));
     TRY(dalloc(sim, &sim->dls, kLsSlots));
+    if (!matrix_free(c)) {
+        sim->splan = plan_solve(g.n_edges, g.P, p.m, c->precision == HDGDG_MIXED);
+        TRY(dalloc(sim, &sim->solve_part, solve_part_bytes(kSolveMaxBlocks) / sizeof(*sim->solve_part)));
+        TRY(dalloc(sim, &sim->solve_epoch, 32));
+        // no value may carry an exchange's number by chance
+        CU(cudaMemsetAsync(sim->solve_part, 0, solve_part_bytes(kSolveMaxBlocks), sim->stream));
+        CU(cudaMemsetAsync(sim->solve_epoch, 0, 32 * sizeof(unsigned), sim->stream));
+        const bool f32 = c->precision == HDGDG_MIXED;
+        void* basis = f32 ? static_cast<void*>(sim->V32) : sim->V;
+        CU(cudaMemsetAsync(basis, 0, basis_vectors(c) * p.nt * (f32 ? sizeof(float) : sizeof(double)), sim->stream));
+    }
     if (!c->host_steps) {
         CU(cudaStreamCreateWithFlags(&sim->body_stream, cudaStreamNonBlocking));
         CU(cudaStreamCreateWithFlags(&sim->side_stream, cudaStreamNonBlocking));
