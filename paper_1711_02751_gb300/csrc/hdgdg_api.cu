@@ -564,18 +564,16 @@ cudaError_t cycle_enqueue(hdgdg_sim* sim, const double* g, cudaStream_t st, bool
     // vectors (w32 holds both): the cycle's first launch zeroes the first, and iteration j's
     // Gram-Schmidt tail zeroes the one product j + 1 adds into.
     const bool fused = kMixed && matrix_free(&sim->cfg) && !sim->ens;
-    cudaError_t e = launch_gmres_cycle_init(ctl, dv_nrm(sim), st);
-    if (e == cudaSuccess) {
-        if constexpr (kMixed) e = launch_scale_by_rnorm(sim->w, dv_nrm(sim), V, n, st, fused ? w : nullptr);
-        else e = launch_scale_by_rnorm(sim->w, dv_nrm(sim), V, n, st);
-    }
-    T* const w_base = w;
     // FP32 matrix-free cycles with Gram-Schmidt twice: the second pass is delayed into the next
     // step (launch_dcgs_fused), whose product is taken of w1 (always in w32's first vector); the
     // products then alternate between the second and third vectors, each zeroed one step ahead
     const bool delayed = fused && sim->cfg.krylov_ortho != 1;
+    cudaError_t e;
+    if constexpr (kMixed)
+        e = launch_cycle_start(ctl, dv_nrm(sim), sim->w, V, n, st, fused ? w : nullptr, delayed ? w + n : nullptr);
+    else e = launch_cycle_start(ctl, dv_nrm(sim), sim->w, V, n, st);
+    T* const w_base = w;
     if constexpr (kMixed) {
-        if (delayed && e == cudaSuccess) e = cudaMemsetAsync(w_base + n, 0, n * sizeof(T), st);
         for (int j = 0; delayed && j < m && e == cudaSuccess; ++j) {
             T* const A = w_base;
             T* const Tj = w_base + (size_t)(1 + (j + 1) % 2) * n;   // this step's product (j >= 1)

@@ -405,10 +405,12 @@ cudaError_t launch_split_pairs_inplace(double* a, size_t n, cudaStream_t s);
 // rotations, residual estimates and the stop flags the loop kernels test.
 struct GmresCtl {
     static constexpr int kM = 32;
-    double H[kM + 1][kM];
-    double Hr[kM + 1][kM];   // the Hessenberg columns before the Givens rotations
-    double cdl[kM + 1];      // H h2 of the last column (launch_dcgs_fused)
-    double cs[kM], sn[kM], s[kM + 1], y[kM];
+    double Hr[kM][kM + 1];       // [column][row]: the Hessenberg columns before the Givens rotations
+    double R[kM][kM + 1];        // [column][row]: after them, and the reciprocals of its diagonal
+    double inv_r[kM];
+    double Q[kM + 1][kM + 1];    // [column][row] of the accumulated rotations
+    double cdl[kM + 1];          // H h2 of the last column (launch_dcgs_fused)
+    double s[kM + 1];
     double tol_abs;     // the solve stops when the residual estimate is <= tol_abs
     double inner_rel;   // a cycle also stops at inner_rel * (its starting residual); 0 = off
     double tol_cycle;
@@ -575,17 +577,16 @@ cudaError_t launch_cycle_end(const double* nrm2, const GmresCtl* ctl, SolveCtl* 
 cudaError_t launch_solve_end(const GmresCtl* ctl, const SolveCtl* sc, StepStats* ss, cudaStream_t s);
 
 cudaError_t launch_gmres_solve_init(GmresCtl* c, double tol_abs, double inner_rel, int maxit, cudaStream_t s);
-cudaError_t launch_gmres_cycle_init(GmresCtl* c, const double* nrm2, cudaStream_t s);
 
-// y = H^{-1} s, then x += V y (FP64 x; V of either type)
+// x += V y, y = R^{-1} s (FP64 x; V of either type)
 cudaError_t launch_gmres_update(const double* V, size_t ldv, GmresCtl* c, double* x, size_t n, cudaStream_t s);
 cudaError_t launch_gmres_update(const float* V, size_t ldv, GmresCtl* c, double* x, size_t n, cudaStream_t s);
-// v = w / sqrt(*nrm2), w in FP64
-cudaError_t launch_scale_by_rnorm(const double* w, const double* nrm2, double* v, size_t n,
-                                  cudaStream_t s);
-// (and zero = 0 when given: the output of the cycle's first fused matrix-free product)
-cudaError_t launch_scale_by_rnorm(const double* w, const double* nrm2, float* v, size_t n,
-                                  cudaStream_t s, float* zero = nullptr);
+// Start a restart cycle from the residual w whose squared norm is *nrm2: the control block and the first
+// basis vector v = w / sqrt(*nrm2) (zero, zero2 = 0 when given: the outputs of the first two fused
+// matrix-free products)
+cudaError_t launch_cycle_start(GmresCtl* c, const double* nrm2, const double* w, double* v, size_t n, cudaStream_t s);
+cudaError_t launch_cycle_start(GmresCtl* c, const double* nrm2, const double* w, float* v, size_t n, cudaStream_t s,
+                               float* zero = nullptr, float* zero2 = nullptr);
 cudaError_t launch_to_f32(const double* a, float* b, size_t n, cudaStream_t s);
 
 // User-state conversion and diagnostics.

@@ -110,19 +110,77 @@ __global__ void split_pairs_inplace_kernel(double* a, size_t n) {
     }
 }
 
-__device__ void gmres_arnoldi_update(GmresCtl* c, int j, int m, const double* h1, const double* h2,
-                                     const double* hn);
+__device__ void gmres_arnoldi_update(GmresCtl* c, int j, int m, const double* h1, const double* h2, double nw1,
+                                     double* hn_out);
 
-// out[j0 + c] = V_{j0+c} . w, c < nj: block partials in scratch, summed by the last block
+// The warp sums of W = 2, 4, 8 or 16 columns at once: at each step of the shuffle tree half the lanes take
+// over half the columns, so that every lane of an FP64 add carries a needed sum -- 16 adds for 16
+// columns, where a tree a column (warp_sum) takes 80, each holding the partition's FP64 pipe for some
+// 60 cycles.  Measured with the two-warp Hessenberg update (219^2, k = 4, mixed form, an Arnoldi step's
+// three passes): 64 -> 47 us; 512^2, k = 3, stiff (two passes): 93 -> 81 us.  The sums and their order
+// are warp_sum's, bit for bit.  Lane l returns column
+// column_of<W>(l).
+template <int W>
+__device__ __forceinline__ int column_of(int lane) {
+    int c = 0;
+#pragma unroll
+    for (int w = W / 2, o = 16; w >= 1; w /= 2, o /= 2) c += (lane & o) ? w : 0;
+    return c;
+}
+
+template <int W>
+__device__ __forceinline__ double warp_sums(double* v, int lane) {
+#pragma unroll
+    for (int w = W / 2, o = 16; o >= 1; w /= 2, o /= 2) {
+        if (w >= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int p = 0; p < W / 2; ++p)
+                if (p < w) {
+                    const double keep = up ? v[p + w] : v[p], give = up ? v[p] : v[p + w];
+                    v[p] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
+    return v[0];
+}
+
+// The sums of NC per-thread values over the block's kDotThreads threads into row[0..NC): warp sums,
+// then the warps in order.
+template <int NC, typename T>
+__device__ __forceinline__ void block_partials(const T* acc, double* row) {
+    __shared__ double sh[NC][kDotThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int c0 = 0; c0 < NC; c0 += 16) {
+        constexpr int kAll = NC < 16 ? NC : 16;
+        constexpr int W = kAll <= 2 ? 2 : kAll <= 4 ? 4 : kAll <= 8 ? 8 : 16;
+        double v[W];
+#pragma unroll
+        for (int q = 0; q < W; ++q) v[q] = c0 + q < NC ? to_f64(acc[c0 + q < NC ? c0 + q : 0]) : 0.0;
+        const double s = warp_sums<W>(v, lane);
+        const int c = c0 + column_of<W>(lane);
+        if (c < NC) sh[c][wid] = s;   // (lanes of one column hold the same sum)
+    }
+    __syncthreads();
+    if (threadIdx.x < NC) {
+        double s = 0.0;
+        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
+        row[threadIdx.x] = s;
+    }
+}
+
+// out[j0 + c] = V_{j0+c} . w, c < CH: block partials in scratch, summed by the last block
 template <int CH, typename T, int VW = 1>
 __global__ void __launch_bounds__(kDotThreads)
-multidot_kernel(const T* __restrict__ V, size_t ldv, int j0, int nj, const T* __restrict__ w,
+multidot_kernel(const T* __restrict__ V, size_t ldv, int j0, const T* __restrict__ w,
                 size_t n, double* __restrict__ scratch, int ldp, double* __restrict__ out,
                 const int* __restrict__ done) {
     if (done && *done) return;
     unsigned* counter = reinterpret_cast<unsigned*>(scratch);
     double* partial = scratch + 1;
-    __shared__ double sh[CH][kDotThreads / 32];
     T acc[CH];
 #pragma unroll
     for (int c = 0; c < CH; ++c) acc[c] = T(0);
@@ -131,40 +189,32 @@ multidot_kernel(const T* __restrict__ V, size_t ldv, int j0, int nj, const T* __
         const Lanes<T, VW> wv = load_lanes<T, VW>(w, iv);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            if (c < nj) {
-                const Lanes<T, VW> v = load_lanes<T, VW>(V + (size_t)(j0 + c) * ldv, iv);
+            const Lanes<T, VW> v = load_lanes<T, VW>(V + (size_t)(j0 + c) * ldv, iv);
 #pragma unroll
-                for (int k = 0; k < VW; ++k) acc[c] += v.v[k] * wv.v[k];
-            }
+            for (int k = 0; k < VW; ++k) acc[c] += v.v[k] * wv.v[k];
         }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        const double s = warp_sum((double)acc[c]);
-        if (lane == 0) sh[c][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < CH && (int)threadIdx.x < nj) {
-        double s = 0.0;
-        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
-        partial[(size_t)blockIdx.x * ldp + j0 + threadIdx.x] = s;
-    }
+    block_partials<CH>(acc, partial + (size_t)blockIdx.x * ldp + j0);
     if (last_block_arrives(counter)) {
-        reduce_partials(partial, gridDim.x, ldp, j0, nj, out + j0);
+        reduce_partials(partial, gridDim.x, ldp, j0, CH, out + j0);
         if (threadIdx.x == 0) *counter = 0u;
     }
 }
 
-// v = w / sqrt(*nrm2) (w in FP64, v in T); zero[idx] = 0 when given
+__device__ void gmres_cycle_init(GmresCtl* c, const double* nrm2);
+
+// Start of a restart cycle: the control block, v = w / sqrt(*nrm2) (w in FP64, v in T); zero = zero2 = 0
+// when given
 template <typename T>
-__global__ void scale_kernel(const double* __restrict__ w, const double* __restrict__ nrm2,
-                             T* __restrict__ v, size_t n, T* __restrict__ zero) {
+__global__ void cycle_start_kernel(GmresCtl* ctl, const double* __restrict__ w, const double* __restrict__ nrm2,
+                                   T* __restrict__ v, size_t n, T* __restrict__ zero, T* __restrict__ zero2) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) gmres_cycle_init(ctl, nrm2);
     const double s = 1.0 / sqrt(*nrm2);
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n;
          idx += (size_t)gridDim.x * blockDim.x) {
         v[idx] = from_f64<T>(w[idx] * s);
         if (zero) zero[idx] = T(0);
+        if (zero2) zero2[idx] = T(0);
     }
 }
 
@@ -189,7 +239,6 @@ axpy_dot_kernel(const T* __restrict__ V, size_t ldv, const double* __restrict__ 
     constexpr int ldp = NJ + 1;
     unsigned* counter = reinterpret_cast<unsigned*>(scratch);
     double* partial = scratch + 1;
-    __shared__ double sh[NJ + 1][kDotThreads / 32];
     T hc[NJ], acc[NJ + 1];
 #pragma unroll
     for (int j = 0; j < NJ; ++j) { hc[j] = T(__ldg(h1 + j)); acc[j] = T(0); }
@@ -214,29 +263,13 @@ axpy_dot_kernel(const T* __restrict__ V, size_t ldv, const double* __restrict__ 
 #pragma unroll
         for (int k = 0; k < VW; ++k) acc[NJ] += x.v[k] * x.v[k];
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c <= NJ; ++c) {
-        const double s = warp_sum((double)acc[c]);
-        if (lane == 0) sh[c][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x <= NJ) {
-        double s = 0.0;
-        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
-        partial[(size_t)blockIdx.x * ldp + threadIdx.x] = s;
-    }
+    block_partials<NJ + 1>(acc, partial + (size_t)blockIdx.x * ldp);
     if (last_block_arrives(counter)) {
         reduce_partials(partial, gridDim.x, ldp, 0, NJ, h2);
         reduce_partials(partial, gridDim.x, ldp, NJ, 1, nw1);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double s2 = *nw1;
-            for (int j = 0; j < NJ; ++j) s2 -= h2[j] * h2[j];
-            *hn = s2 > 0.0 ? sqrt(s2) : 0.0;
-            if (ctl) gmres_arnoldi_update(ctl, jcol, m, h1, h2, hn);
-            *counter = 0u;
-        }
+        if (threadIdx.x < 64) gmres_arnoldi_update(ctl, jcol, m, h1, h2, *nw1, hn);
+        if (threadIdx.x == 0) *counter = 0u;
     }
 }
 
@@ -304,7 +337,6 @@ dcgs_fused_kernel(const T* __restrict__ V, size_t ldv, const double* __restrict_
     constexpr int ldp = NJ + 1;
     unsigned* counter = reinterpret_cast<unsigned*>(scratch);
     double* partial = scratch + 1;
-    __shared__ double sh[NJ + 1][kDotThreads / 32];
     T a[NJ], cc[NJ + 1], acc[NJ + 1];
 #pragma unroll
     for (int j = 0; j < NJ; ++j) a[j] = T(__ldg(h2 + j));
@@ -344,18 +376,7 @@ dcgs_fused_kernel(const T* __restrict__ V, size_t ldv, const double* __restrict_
 #pragma unroll
         for (int k = 0; k < VW; ++k) acc[NJ] += x.v[k] * y.v[k];
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c <= NJ; ++c) {
-        const double s = warp_sum((double)acc[c]);
-        if (lane == 0) sh[c][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x <= NJ) {
-        double s = 0.0;
-        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
-        partial[(size_t)blockIdx.x * ldp + threadIdx.x] = s;
-    }
+    block_partials<NJ + 1>(acc, partial + (size_t)blockIdx.x * ldp);
     if (last_block_arrives(counter)) {
         reduce_partials(partial, gridDim.x, ldp, 0, NJ + 1, h1n);
         if (threadIdx.x == 0) *counter = 0u;
@@ -371,7 +392,6 @@ __device__ __forceinline__ void guess_norms_body(size_t n, const double* __restr
     constexpr int NQ = 7;
     unsigned* counter = reinterpret_cast<unsigned*>(scratch);
     double* partial = scratch + 1;
-    __shared__ double sh[NQ][kDotThreads / 32];
     double acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
@@ -392,18 +412,7 @@ __device__ __forceinline__ void guess_norms_body(size_t n, const double* __restr
             acc[q] += r * r;
         }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const double s = warp_sum(acc[q]);
-        if (lane == 0) sh[q][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < NQ) {
-        double s = 0.0;
-        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
-        partial[(size_t)blockIdx.x * NQ + threadIdx.x] = s;
-    }
+    block_partials<NQ>(acc, partial + (size_t)blockIdx.x * NQ);
     if (last_block_arrives(counter)) {
         reduce_partials(partial, gridDim.x, NQ, 0, NQT + 1, out);
         if (threadIdx.x == 0) *counter = 0u;
@@ -423,7 +432,6 @@ __device__ __forceinline__ void guess_norms_x2_body(size_t n, const double* __re
     constexpr int NQ = 7;
     unsigned* counter = reinterpret_cast<unsigned*>(scratch);
     double* partial = scratch + 1;
-    __shared__ double sh[NQ][kDotThreads / 32];
     __shared__ float cf[NQ][6];   // c[q][j] (binomial coefficients: exact in FP32)
     if (threadIdx.x < NQ * 6) cf[threadIdx.x / 6][threadIdx.x % 6] = f64_to_f32(t.c[threadIdx.x / 6][threadIdx.x % 6]);
     __syncthreads();
@@ -464,18 +472,7 @@ __device__ __forceinline__ void guess_norms_x2_body(size_t n, const double* __re
             }
         }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const double s = warp_sum(f32_to_f64(acc[q]));
-        if (lane == 0) sh[q][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < NQ) {
-        double s = 0.0;
-        for (int k = 0; k < kDotThreads / 32; ++k) s += sh[threadIdx.x][k];
-        partial[(size_t)blockIdx.x * NQ + threadIdx.x] = s;
-    }
+    block_partials<NQ>(acc, partial + (size_t)blockIdx.x * NQ);
     if (last_block_arrives(counter)) {
         reduce_partials(partial, gridDim.x, NQ, 0, NQT + 1, out);
         if (threadIdx.x == 0) *counter = 0u;
@@ -697,57 +694,76 @@ __global__ void gmres_solve_init_kernel(GmresCtl* c, double tol_abs, double inne
     c->status = 0;
 }
 
-// Start a restart cycle from the residual whose squared norm is *nrm2.
-__global__ void gmres_cycle_init_kernel(GmresCtl* c, const double* nrm2) {
+// Start a restart cycle from the residual whose squared norm is *nrm2 (one thread).
+__device__ void gmres_cycle_init(GmresCtl* c, const double* nrm2) {
     const double rn = sqrt(*nrm2);
     c->rnorm = rn;
     for (int i = 0; i <= GmresCtl::kM; ++i) c->s[i] = 0.0;
     c->s[0] = rn;
+    c->Q[0][0] = 1.0;
     c->jend = 0;
     c->done = c->total >= c->maxit ? 1 : 0;
     c->tol_cycle = fmax(c->tol_abs, c->inner_rel * rn);
 }
 
-// Column j of the Hessenberg matrix from the two Gram-Schmidt passes, Givens rotations, the
-// residual estimate |s_{j+1}| and the cycle's stop test (one thread).
-__device__ void gmres_arnoldi_update(GmresCtl* c, int j, int m, const double* h1, const double* h2,
-                                     const double* hn) {
-    if (c->done) return;
-    for (int i = 0; i <= j; ++i) c->H[i][j] = c->Hr[i][j] = h1[i] + h2[i];
-    c->H[j + 1][j] = c->Hr[j + 1][j] = *hn;
-    // c = H h2 over the raw columns 0..j (the delayed second pass's correction of the next product)
-    for (int i = 0; i <= j + 1; ++i) {
+// Column j of the Hessenberg matrix from the two Gram-Schmidt passes, hn = sqrt(||w1||^2 - ||h2||^2),
+// the rotations, the residual estimate |s_{j+1}| and the cycle's stop test, by two warps, lane i
+// holding row i: warp 0 the column and c = H h2 (the delayed second pass's correction of the next
+// product), warp 1 the accumulated rotations applied to the column and the new one.  (One thread
+// went through some 250 dependent FP64 operations and as many loads.)  No control block: hn alone.
+__device__ void gmres_arnoldi_update(GmresCtl* c, int j, int m, const double* h1, const double* h2, double nw1,
+                                     double* hn_out) {
+    const int lane = threadIdx.x & 31;
+    const bool first = threadIdx.x < 32;
+    const double h2v = lane <= j ? h2[lane] : 0.0;
+    double s2 = nw1;
+    for (int k = 0; k <= j; ++k) {
+        const double h = __shfl_sync(0xffffffffu, h2v, k);
+        s2 -= h * h;
+    }
+    const double hn = s2 > 0.0 ? sqrt(s2) : 0.0;
+    if (first && lane == 0) *hn_out = hn;
+    if (!c || c->done) return;   // (done is set below only after both warps' reads: see the barrier)
+    const double hc = lane <= j ? h1[lane] + h2v : 0.0;
+    if (first) {
+        const double col = lane == j + 1 ? hn : hc;
         double t = 0.0;
-        for (int k = i > 0 ? i - 1 : 0; k <= j; ++k) t += c->Hr[i][k] * h2[k];
-        c->cdl[i] = t;
+#pragma unroll 8
+        for (int k = 0; k < j; ++k) t += c->Hr[k][lane] * __shfl_sync(0xffffffffu, h2v, k);
+        t += col * __shfl_sync(0xffffffffu, h2v, j);
+        c->Hr[j][lane] = col;
+        c->cdl[lane] = t;
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        return;
     }
-    for (int i = 0; i < j; ++i) {
-        const double t = c->cs[i] * c->H[i][j] + c->sn[i] * c->H[i + 1][j];
-        c->H[i + 1][j] = -c->sn[i] * c->H[i][j] + c->cs[i] * c->H[i + 1][j];
-        c->H[i][j] = t;
+    double r = 0.0;
+#pragma unroll 8
+    for (int k = 0; k <= j; ++k) r += c->Q[k][lane] * __shfl_sync(0xffffffffu, hc, k);
+    const double a = __shfl_sync(0xffffffffu, r, j);
+    const double den = sqrt(a * a + hn * hn);
+    const double inv = 1.0 / den;
+    const double cs = den > 0.0 ? a * inv : 1.0, sn = den > 0.0 ? hn * inv : 0.0;
+    c->R[j][lane] = lane < j ? r : lane == j ? den : 0.0;
+    if (lane <= j) {
+        const double qv = c->Q[lane][j];
+        c->Q[lane][j] = cs * qv;
+        c->Q[lane][j + 1] = -sn * qv;
     }
-    const double a = c->H[j][j], b = c->H[j + 1][j];
-    const double den = hypot(a, b);
-    const double cs = den > 0.0 ? a / den : 1.0, sn = den > 0.0 ? b / den : 0.0;
-    c->cs[j] = cs;
-    c->sn[j] = sn;
-    c->H[j][j] = den;
-    c->H[j + 1][j] = 0.0;
-    c->s[j + 1] = -sn * c->s[j];
-    c->s[j] = cs * c->s[j];
-    c->total += 1;
-    c->jend = j + 1;
-    const double est = fabs(c->s[j + 1]);
-    if (!isfinite(est)) { c->status = 1; c->done = 1; return; }
-    if (est <= c->tol_cycle || b == 0.0 || c->total >= c->maxit || j == m - 1) c->done = 1;
-}
-
-// y = H(0:jend, 0:jend)^{-1} s by back substitution.
-__global__ void gmres_solve_y_kernel(GmresCtl* c) {
-    for (int i = c->jend - 1; i >= 0; --i) {
-        double acc = c->s[i];
-        for (int k = i + 1; k < c->jend; ++k) acc -= c->H[i][k] * c->y[k];
-        c->y[i] = acc / c->H[i][i];
+    c->Q[j + 1][lane] = lane == j ? sn : lane == j + 1 ? cs : 0.0;
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+    if (lane == 0) {
+        const double sj = c->s[j], est = fabs(sn * sj);
+        c->s[j + 1] = -sn * sj;
+        c->s[j] = cs * sj;
+        c->inv_r[j] = inv;
+        c->total += 1;
+        c->jend = j + 1;
+        if (!isfinite(est)) {
+            c->status = 1;
+            c->done = 1;
+        } else if (est <= c->tol_cycle || hn == 0.0 || c->total >= c->maxit || j == m - 1) {
+            c->done = 1;
+        }
     }
 }
 
@@ -755,13 +771,21 @@ __global__ void gmres_solve_y_kernel(GmresCtl* c) {
 // cycles): the correction is summed in FP32 -- the cycle that produced it is FP32 throughout --
 // and added to the FP64 iterate once, one conversion (fastcvt.h) and one FP64 add per entry.
 // VW entries per thread (16-byte lanes of FP32 bases); the basis loads are issued four vectors at a
-// time and added in their order.
+// time and added in their order.  Each block's first warp solves R y = s itself (lane i holding row i).
 template <typename T, int VW = 1>
 __global__ void gmres_update_x_kernel(const T* __restrict__ V, size_t ldv, const GmresCtl* __restrict__ c,
                                       double* __restrict__ x, size_t n) {
     const int nv = c->jend;
     __shared__ T sy[GmresCtl::kM];
-    for (int j = threadIdx.x; j < nv; j += blockDim.x) sy[j] = T(c->y[j]);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        double s = lane < nv ? c->s[lane] : 0.0;
+        for (int i = nv - 1; i >= 0; --i) {
+            const double y = __shfl_sync(0xffffffffu, s, i) * c->inv_r[i];
+            if (lane == 0) sy[i] = T(y);
+            if (lane < i) s -= c->R[i][lane] * y;
+        }
+    }
     __syncthreads();
     for (size_t iv = blockIdx.x * (size_t)blockDim.x + threadIdx.x; iv < n / VW;
          iv += (size_t)gridDim.x * blockDim.x) {
@@ -920,18 +944,16 @@ cudaError_t multidot_impl(const T* V, size_t ldv, int nv, const T* w, size_t n, 
     case C:                                                                                                       \
         if constexpr (sizeof(T) == 4) {                                                                           \
             if (v4) {                                                                                             \
-                multidot_kernel<C, T, 4><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, nj, w, n, scratch, nv, out, \
-                                                                           done);                                 \
+                multidot_kernel<C, T, 4><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, w, n, scratch, nv, out, done); \
                 break;                                                                                            \
             }                                                                                                     \
         } else {                                                                                                  \
             if (v2) {                                                                                             \
-                multidot_kernel<C, T, 2><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, nj, w, n, scratch, nv, out, \
-                                                                           done);                                 \
+                multidot_kernel<C, T, 2><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, w, n, scratch, nv, out, done); \
                 break;                                                                                            \
             }                                                                                                     \
         }                                                                                                         \
-        multidot_kernel<C, T><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, nj, w, n, scratch, nv, out, done);   \
+        multidot_kernel<C, T><<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, j0, w, n, scratch, nv, out, done);   \
         break;
             CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
@@ -1078,16 +1100,15 @@ cudaError_t launch_multidot(const float* V, size_t ldv, int nv, const float* w, 
     return multidot_impl<float>(V, ldv, nv, w, n, scratch, out, s, done);
 }
 
-cudaError_t launch_scale_by_rnorm(const double* w, const double* nrm2, double* v, size_t n,
-                                  cudaStream_t s) {
-    scale_kernel<double><<<stream_grid(n), 256, 0, s>>>(w, nrm2, v, n, nullptr);
+cudaError_t launch_cycle_start(GmresCtl* c, const double* nrm2, const double* w, double* v, size_t n, cudaStream_t s) {
+    cycle_start_kernel<double><<<stream_grid(n), 256, 0, s>>>(c, w, nrm2, v, n, nullptr, nullptr);
     count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_by_rnorm(const double* w, const double* nrm2, float* v, size_t n,
-                                  cudaStream_t s, float* zero) {
-    scale_kernel<float><<<stream_grid(n), 256, 0, s>>>(w, nrm2, v, n, zero);
+cudaError_t launch_cycle_start(GmresCtl* c, const double* nrm2, const double* w, float* v, size_t n, cudaStream_t s,
+                               float* zero, float* zero2) {
+    cycle_start_kernel<float><<<stream_grid(n), 256, 0, s>>>(c, w, nrm2, v, n, zero, zero2);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1098,25 +1119,16 @@ cudaError_t launch_gmres_solve_init(GmresCtl* c, double tol_abs, double inner_re
     return cudaGetLastError();
 }
 
-cudaError_t launch_gmres_cycle_init(GmresCtl* c, const double* nrm2, cudaStream_t s) {
-    gmres_cycle_init_kernel<<<1, 1, 0, s>>>(c, nrm2);
+cudaError_t launch_gmres_update(const double* V, size_t ldv, GmresCtl* c, double* x, size_t n, cudaStream_t s) {
+    gmres_update_x_kernel<double><<<stream_grid(n), 256, 0, s>>>(V, ldv, c, x, n);
     count_launches(1);
     return cudaGetLastError();
 }
 
-
-cudaError_t launch_gmres_update(const double* V, size_t ldv, GmresCtl* c, double* x, size_t n, cudaStream_t s) {
-    gmres_solve_y_kernel<<<1, 1, 0, s>>>(c);
-    gmres_update_x_kernel<double><<<stream_grid(n), 256, 0, s>>>(V, ldv, c, x, n);
-    count_launches(2);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_gmres_update(const float* V, size_t ldv, GmresCtl* c, double* x, size_t n, cudaStream_t s) {
-    gmres_solve_y_kernel<<<1, 1, 0, s>>>(c);
     if (lanes4<float>(n, ldv, {V})) gmres_update_x_kernel<float, 4><<<stream_grid(n / 4), 256, 0, s>>>(V, ldv, c, x, n);
     else gmres_update_x_kernel<float><<<stream_grid(n), 256, 0, s>>>(V, ldv, c, x, n);
-    count_launches(2);
+    count_launches(1);
     return cudaGetLastError();
 }
 

@@ -34,7 +34,7 @@
 // between them at small sizes, S~'s bytes through 448 threads an SM at large ones.
 #include <cstdint>
 
-#include "compensated.h"
+#include "pairsum.h"
 #include "solve.h"
 
 namespace hdgdg {
@@ -44,42 +44,6 @@ constexpr int kNT = kSolveThreads, kNW = kNT / 32;
 constexpr int kCtlWarps = 2;                    // warps 0 and 1: Hessenberg column, rotation, stop test
 constexpr int kProdThreads = kNT - 32 * kCtlWarps;
 constexpr unsigned kMaxSpins = 1u << 22;        // bound of every wait
-
-// A sum across lanes: FP64, or an FP32 pair (hi + lo, |lo| <= ulp(hi) / 2).
-struct PairSum {
-    float hi, lo;
-};
-__device__ __forceinline__ PairSum add(PairSum a, PairSum b) {
-    float s, e;
-    two_sum(a.hi, b.hi, s, e);
-    e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-    PairSum r;
-    r.hi = __fadd_rn(s, e);
-    r.lo = __fsub_rn(e, __fsub_rn(r.hi, s));
-    return r;
-}
-__device__ __forceinline__ PairSum add(PairSum a, float b) {
-    float s, e;
-    two_sum(a.hi, b, s, e);
-    return PairSum{s, __fadd_rn(a.lo, e)};
-}
-__device__ __forceinline__ double add(double a, double b) { return a + b; }
-__device__ __forceinline__ PairSum shfl_xor(PairSum v, int o) {
-    return PairSum{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-}
-__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ double value(PairSum v) { return f32_to_f64(v.hi) + f32_to_f64(v.lo); }
-__device__ __forceinline__ double value(double v) { return v; }
-template <typename T>   // double
-struct SumOf {
-    using S = double;
-    static __device__ __forceinline__ S of(T v) { return v; }
-};
-template <>
-struct SumOf<float> {
-    using S = PairSum;
-    static __device__ __forceinline__ S of(float v) { return PairSum{v, 0.f}; }
-};
 
 // Values that cross blocks: each 32-bit half in an 8-byte word (accessed at once) under the 32-bit
 // number of the exchange it belongs to.

@@ -7,7 +7,7 @@ stop test: 1e-9 ||g|| in the mixed form (its residual is FP64-class, 1e-13), the
 FP64 form.  Sizes: fewer edges than one block takes, a ragged last block, every split of a row's
 columns (k = 1..8), restart lengths 1 and 31, absent sides and prescribed traces, an FP32 basis that
 all but fills shared memory (128^2, k = 3) and the first size past it, which keeps the
-launch-per-operation path."""
+launch-per-operation path; there restart lengths that cover every width of its column reductions."""
 import numpy as np
 import pytest
 
@@ -18,6 +18,7 @@ hd = pytest.importorskip("paper_1711_02751_gb300.hdgdg")
 
 FAST = dict(precision="mixed", local_precision="f32x2", residual_f32x2=True)
 MIXED = dict(precision="mixed")
+MF = dict(precision="mixed", local_precision="f32x2", trace_operator=1)
 V = W.VORTEX
 VORTEX = dict(boundary="vortex", x0=-2.0, length=4.0, g=V["g"], H0=V["H_inf"],
               bc_params=(V["beta"], V["u_inf"], V["v_inf"], V["xc"], V["yc"]))
@@ -29,7 +30,9 @@ VORTEX = dict(boundary="vortex", x0=-2.0, length=4.0, g=V["g"], H0=V["H_inf"],
     (2, 2, FAST), (33, 2, FAST), (12, 1, FAST), (47, 4, FAST), (20, 5, MIXED), (11, 6, FAST), (13, 7, FAST),
     (9, 8, FAST), (6, 3, dict(FAST, boundary="wall")), (6, 4, dict(FAST, **VORTEX)),
     (24, 3, dict(FAST, krylov_restart=1)), (24, 2, dict(MIXED, krylov_restart=31)),
-    (40, 3, dict(FAST, krylov_ortho=1)), (128, 3, FAST), (160, 3, FAST)])
+    (40, 3, dict(FAST, krylov_ortho=1)), (128, 3, FAST), (160, 3, FAST),
+    # the launch-per-operation path: reductions of up to 32 columns at once, and the FP64 form's
+    (24, 3, dict(MF, krylov_restart=31)), (15, 2, dict(MF, krylov_restart=3)), (120, 3, dict(krylov_restart=31))])
 def test_solution_satisfies_the_trace_system(N, k, kw):
     rng = np.random.default_rng(N * 10 + k)
     kw = dict(kw)
