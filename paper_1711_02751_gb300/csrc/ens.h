@@ -21,6 +21,29 @@ __device__ __forceinline__ void ens_walk(const EnsTable& t, F&& body) {
     }
 }
 
+// The mesh numbers of a group (periodic) as values of their own: the compiler keeps the few that a body
+// uses in registers, all loaded at once when the item starts, instead of reading the group's Geom in
+// device memory wherever the connectivity needs it.  The GLL tables stay behind.
+__device__ __forceinline__ Geom ens_mesh(const EnsGroup& G) {
+    Geom g;
+    g.N = G.g.N;
+    g.P = G.g.P;
+    g.Np = G.g.Np;
+    g.n_el = G.g.n_el;
+    g.n_edges = G.g.n_edges;
+    g.batch = G.g.batch;
+    g.n_el_inst = G.g.n_el_inst;
+    g.n_edges_inst = G.g.n_edges_inst;
+    g.dt_scale = G.g.dt_scale;
+    g.walls = 0;
+    g.dirichlet = 0;
+    g.byN = G.g.byN;
+    g.byN1 = G.g.byN1;
+    g.by_el = G.g.by_el;
+    g.by_edges = G.g.by_edges;
+    return g;
+}
+
 // The launch table for a kind of work: blocks(group) blocks for each group.
 template <class Blocks>
 EnsTable ens_table(const EnsHost& E, Blocks blocks) {

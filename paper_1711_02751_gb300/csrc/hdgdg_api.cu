@@ -563,11 +563,11 @@ cudaError_t cycle_enqueue(hdgdg_sim* sim, const double* g, cudaStream_t st, bool
     // The fused matrix-free product adds into its output, so the products alternate between two
     // vectors (w32 holds both): the cycle's first launch zeroes the first, and iteration j's
     // Gram-Schmidt tail zeroes the one product j + 1 adds into.
-    const bool fused = kMixed && matrix_free(&sim->cfg) && !sim->ens;
+    const bool fused = kMixed && matrix_free(&sim->cfg);
     // FP32 matrix-free cycles with Gram-Schmidt twice: the second pass is delayed into the next
     // step (launch_dcgs_fused), whose product is taken of w1 (always in w32's first vector); the
     // products then alternate between the second and third vectors, each zeroed one step ahead
-    const bool delayed = fused && sim->cfg.krylov_ortho != 1;
+    const bool delayed = fused && !sim->ens && sim->cfg.krylov_ortho != 1;
     cudaError_t e;
     if constexpr (kMixed)
         e = launch_cycle_start(ctl, dv_nrm(sim), sim->w, V, n, st, fused ? w : nullptr, delayed ? w + n : nullptr);
@@ -598,7 +598,7 @@ cudaError_t cycle_enqueue(hdgdg_sim* sim, const double* g, cudaStream_t st, bool
         {
             TimedGroup tg(sim, HDGDG_KT_SPMV, j);
             if constexpr (kMixed) {
-                if (sim->ens) e = launch_ens_mf_inner(*sim->ens, sim->mf, n, Vj, w, st, done);
+                if (sim->ens) e = launch_ens_mf_inner(*sim->ens, Vj, w, st, done);
                 else if (fused) e = launch_mf_inner(sim->g, sim->mf, Vj, w, beta_of(sim), st, done, true);
                 else
                     e = launch_spmv_pre(sim->g, St, sim->Scol, Vj, w, st, done,
@@ -2192,7 +2192,7 @@ hdgdg_status ens_super(hdgdg_ensemble* E, const hdgdg_config* base, size_t n_tot
             TRY(dalloc(sim, &sim->yhist[i][h], p.nt));
         }
     TRY(dalloc(sim, &sim->V32, (size_t)(p.m + 1) * p.nt));
-    TRY(dalloc(sim, &sim->w32, p.nt));
+    TRY(dalloc(sim, &sim->w32, 2 * p.nt));   // two alternating product outputs
     TRY(dalloc(sim, &sim->red, reduction_scratch_doubles(p.m, edges_total, 3)));
     CU(cudaMemset(sim->red, 0, sizeof(double)));
     TRY(dalloc(sim, &sim->mred, mass_scratch_doubles()));
@@ -2213,6 +2213,10 @@ hdgdg_status ens_super(hdgdg_ensemble* E, const hdgdg_config* base, size_t n_tot
     sim->mf.ybuf = ybuf;
     sim->mf.hm = hm;
     sim->mf.hp = hp;
+    // the values between the groups' slices take part in the vector operations as zeros
+    for (double* v : {sim->gvec, sim->xt, sim->lam, sim->w, ybuf, hm, hp}) CU(cudaMemsetAsync(v, 0, p.nt * sizeof(double), sim->stream));
+    CU(cudaMemsetAsync(sim->V32, 0, (size_t)(p.m + 1) * p.nt * sizeof(float), sim->stream));
+    CU(cudaMemsetAsync(sim->w32, 0, 2 * p.nt * sizeof(float), sim->stream));
     CU(cudaMemsetAsync(sim->flags, 0, 16, sim->stream));
     CU(cudaStreamSynchronize(sim->stream));
     return HDGDG_OK;
@@ -2290,6 +2294,8 @@ hdgdg_status hdgdg_ensemble_create(const hdgdg_config* base, int n_members, cons
         G.beta = beta_of(gs);
         G.phiB = gs->phiB;
         G.tau = gs->tau;
+        G.tau32 = gs->mf.tau32;
+        G.tau2 = gs->mf.tau2;
         G.S2 = gs->ops.S;
         G.aux2 = gs->ops.aux;
         G.EG2 = gs->ops.EG;
@@ -2298,9 +2304,9 @@ hdgdg_status hdgdg_ensemble_create(const hdgdg_config* base, int n_members, cons
         G.EG32 = gs->mf.EG32;
         G.Minv = gs->mf.Minv;
         off3 += 3 * gs->plan.n;
-        offt += gs->plan.nt;
+        offt = (offt + gs->plan.nt + 3) & ~(size_t)3;   // 16-byte slices of FP32 vectors
         n_total += gs->plan.n;
-        nt_total += gs->plan.nt;
+        nt_total = offt;
         edges_total += gs->g.n_edges;
     }
     E->host.ngroups = (int)keys.size();

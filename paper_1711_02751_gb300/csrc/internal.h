@@ -479,10 +479,13 @@ cudaError_t launch_dcgs_fused(const float* V, size_t ldv, int nj, const double* 
 constexpr int kEnsMaxGroups = 32;
 struct EnsGroup {
     Geom g;                     // the group's mesh (a batch of same-size instances)
-    size_t off3, offt;          // its slice: state vectors (3 fields), trace vectors
+    size_t off3, offt;          // its slice: state vectors (3 fields), trace vectors (offt a multiple of 4;
+                                // the values between the slices stay zero)
     double dt, beta;            // its time step and lift factor dt a_ii (2/h) / w_0
     const double* phiB;
     const double* tau;
+    const float* tau32;                   // tau_hat in FP32 (the inner product) and as FP32 pairs
+    const void* tau2;
     const void *S2, *aux2, *EG2;          // Schur-complement operators as FP32 pairs
     const float *S32, *aux32, *EG32;      // and as FP32 (the inner cycles)
     PrecondBlocks Minv;                   // block-Jacobi inverse, FP16 blocks and scales
@@ -504,9 +507,9 @@ cudaError_t launch_ens_condense(const EnsHost& E, const double* R1, double* Z, d
 // recovery: Q = Z + beta A^{-1}(tau qhat), Lst = (Q - R1)/a_ii
 cudaError_t launch_ens_recover(const EnsHost& E, const double* Z, const double* R1, const double* qhat,
                                double inv_aii, double* Q, double* Lst, cudaStream_t s);
-// matrix-free trace operator over every group: inner (FP32), residual (FP32 pairs), back-transformation
-cudaError_t launch_ens_mf_inner(const EnsHost& E, const MfOps& scratch, size_t nt, const float* x, float* y,
-                                cudaStream_t s, const int* done);
+// matrix-free trace operator over every group: inner (FP32; adds into y, zero beforehand), residual
+// (FP32 pairs), back-transformation
+cudaError_t launch_ens_mf_inner(const EnsHost& E, const float* x, float* y, cudaStream_t s, const int* done);
 cudaError_t launch_ens_mf_residual(const EnsHost& E, const MfOps& scratch, size_t nt, const double* x,
                                    const double* rhs, double* w, cudaStream_t s);
 cudaError_t launch_ens_mf_back(const EnsHost& E, const double* x, double* y, cudaStream_t s);

@@ -614,22 +614,39 @@ __global__ void __launch_bounds__(256) ens_mf_pre_kernel(EnsTable t, const TX* _
     });
 }
 
+// The refinement residual's element pass, and (the inner product) the fused pass: y = M^{-1} x on each
+// face in shared memory, both sides added into the zeroed output (mf_elem_body).
+template <int P, class A, int MODE>
+__device__ __forceinline__ void ens_mf_elem_item(const EnsGroup& G, int bid, const MfVec<MODE>* x, const void* y,
+                                                 MfVec<MODE>* hm, MfVec<MODE>* hp) {
+    using T = typename A::T;
+    const Geom g = ens_mesh(G);
+    const size_t o = G.offt;
+    if constexpr (MODE == kMfInner)
+        mf_elem_body<P, mf_epb<P>(), A, MODE, false, true>(bid, g, G.S32, G.aux32, G.EG32, G.tau32, x + o, hm + o,
+                                                          nullptr, G.beta, G.Minv);
+    else
+        mf_elem_body<P, mf_epb<P>(), A, MODE, false, false, true>(
+            bid, g, static_cast<const T*>(G.S2), static_cast<const T*>(G.aux2), static_cast<const T*>(G.EG2), G.tau2,
+            static_cast<const T*>(y) + o, hm + o, hp + o, G.beta);
+}
+
+// The three degrees' bodies in one kernel take 128 registers a thread (the residual 208, one block an SM)
+// unless they are capped: six blocks an SM for the inner product, four for the residual, the operator
+// loaded where it is used.  24 members (16^2 to 128^2, k = 2..4, 130 560 elements): the product in one
+// launch at two blocks an SM took no less than the three it replaces (17.1 ms a step), at 3 / 4 / 5 / 6
+// blocks 15.1 / 15.4 / 12.4 / 12.0 ms a step; 128-thread blocks 13.3 at eight an SM.
 template <class A, int MODE>
-__global__ void __launch_bounds__(256) ens_mf_elem_kernel(EnsTable t, const typename A::T* __restrict__ y,
+__global__ void __launch_bounds__(256, MODE == kMfInner ? 6 : 4) ens_mf_elem_kernel(EnsTable t, const MfVec<MODE>* __restrict__ x,
+                                                          const typename A::T* __restrict__ y,
                                                           MfVec<MODE>* __restrict__ hm, MfVec<MODE>* __restrict__ hp,
                                                           const int* __restrict__ done) {
     if (done && *done) return;
-    constexpr bool k32 = sizeof(typename A::T) == sizeof(float);
     ens_walk(t, [&](const EnsGroup& G, int bid) {
-        using T = typename A::T;
-        const T* S = k32 ? reinterpret_cast<const T*>(G.S32) : static_cast<const T*>(G.S2);
-        const T* aux = k32 ? reinterpret_cast<const T*>(G.aux32) : static_cast<const T*>(G.aux2);
-        const T* EG = k32 ? reinterpret_cast<const T*>(G.EG32) : static_cast<const T*>(G.EG2);
-        const size_t o = G.offt;
         switch (G.g.P) {
-            case 3: mf_elem_body<3, mf_epb<3>(), A, MODE, true>(bid, G.g, S, aux, EG, G.tau, y + o, hm + o, hp + o, G.beta); break;
-            case 4: mf_elem_body<4, mf_epb<4>(), A, MODE, true>(bid, G.g, S, aux, EG, G.tau, y + o, hm + o, hp + o, G.beta); break;
-            case 5: mf_elem_body<5, mf_epb<5>(), A, MODE, true>(bid, G.g, S, aux, EG, G.tau, y + o, hm + o, hp + o, G.beta); break;
+            case 3: ens_mf_elem_item<3, A, MODE>(G, bid, x, y, hm, hp); break;
+            case 4: ens_mf_elem_item<4, A, MODE>(G, bid, x, y, hm, hp); break;
+            case 5: ens_mf_elem_item<5, A, MODE>(G, bid, x, y, hm, hp); break;
             default: break;
         }
     });
@@ -654,24 +671,6 @@ int ens_edge_blocks(const EnsGroup& G) {
 int ens_mf_elem_blocks(const EnsGroup& G) {
     const int P = G.g.P, epb = 256 / (P * P) > 32 ? 32 : 256 / (P * P);
     return (G.g.n_el + epb - 1) / epb;
-}
-
-template <class A, int MODE>
-cudaError_t ens_mf_launch(const EnsHost& E, const MfOps& op, size_t nt, const MfVec<MODE>* x, const double* rhs,
-                          MfVec<MODE>* out, cudaStream_t s, const int* done) {
-    using T = typename A::T;
-    using TO = MfVec<MODE>;
-    const EnsTable te = ens_table(E, ens_edge_blocks);
-    const EnsTable tm = ens_table(E, ens_mf_elem_blocks);
-    T* y = static_cast<T*>(op.ybuf);
-    TO* hm = static_cast<TO*>(op.hm);
-    TO* hp = static_cast<TO*>(op.hp);
-    ens_mf_pre_kernel<A, TO><<<ens_grid(ens_mf_pre_kernel<A, TO>, te.start[te.ngroups]), 256, 0, s>>>(te, x, y, done);
-    ens_mf_elem_kernel<A, MODE><<<ens_grid(ens_mf_elem_kernel<A, MODE>, tm.start[tm.ngroups]), 256, 0, s>>>(tm, y, hm,
-                                                                                                         hp, done);
-    mf_sum_kernel<TO, MODE == kMfResidual><<<sum_grid(nt), 256, 0, s>>>(nt, hm, hp, rhs, out, done);
-    count_launches(3);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -779,14 +778,31 @@ void mf_tile_info(int P, int t, int* epb, int* prefetch) {
     *prefetch = mf_tile_pref(t) ? 1 : 0;
 }
 
-cudaError_t launch_ens_mf_inner(const EnsHost& E, const MfOps& scratch, size_t nt, const float* x, float* y,
-                                cudaStream_t s, const int* done) {
-    return ens_mf_launch<ArithF32, kMfInner>(E, scratch, nt, x, nullptr, y, s, done);
+cudaError_t launch_ens_mf_inner(const EnsHost& E, const float* x, float* y, cudaStream_t s, const int* done) {
+    // the fused pass's vector loads (3(k + 1) a multiple of 4): x on 16 bytes, the FP16 blocks on 8
+    for (int i = 0; i < E.ngroups; ++i)
+        if ((3 * E.h[i].g.P) % 4 == 0 && (reinterpret_cast<uintptr_t>(x + E.h[i].offt) % 16 != 0 ||
+                                          reinterpret_cast<uintptr_t>(E.h[i].Minv.h) % 8 != 0))
+            return cudaErrorMisalignedAddress;
+    const EnsTable tm = ens_table(E, ens_mf_elem_blocks);
+    const auto k = ens_mf_elem_kernel<ArithF32, kMfInner>;
+    k<<<ens_grid(k, tm.start[tm.ngroups]), 256, 0, s>>>(tm, x, nullptr, y, nullptr, done);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ens_mf_residual(const EnsHost& E, const MfOps& scratch, size_t nt, const double* x,
                                    const double* rhs, double* w, cudaStream_t s) {
-    return ens_mf_launch<ArithF2, kMfResidual>(E, scratch, nt, x, rhs, w, s, nullptr);
+    const EnsTable te = ens_table(E, ens_edge_blocks), tm = ens_table(E, ens_mf_elem_blocks);
+    float2* y = static_cast<float2*>(scratch.ybuf);
+    double *hm = static_cast<double*>(scratch.hm), *hp = static_cast<double*>(scratch.hp);
+    const auto kp = ens_mf_pre_kernel<ArithF2, double>;
+    const auto ke = ens_mf_elem_kernel<ArithF2, kMfResidual>;
+    kp<<<ens_grid(kp, te.start[te.ngroups]), 256, 0, s>>>(te, x, y, nullptr);
+    ke<<<ens_grid(ke, tm.start[tm.ngroups]), 256, 0, s>>>(tm, nullptr, y, hm, hp, nullptr);
+    mf_sum_kernel<double, true><<<sum_grid(nt), 256, 0, s>>>(nt, hm, hp, rhs, w, nullptr);
+    count_launches(3);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ens_mf_back(const EnsHost& E, const double* x, double* y, cudaStream_t s) {
