@@ -136,7 +136,7 @@ Plan make_plan(const hdgdg_config* c) {
     if (c->precision == HDGDG_MIXED && c->residual_f32x2 && !matrix_free(c))
         b += n_edges * 6 * (size_t)p.NF * p.NF * sizeof(float);
     if (matrix_free(c)) {   // FP16 M^{-1} and scales, FP32 Schur operators, the operator's scratch
-        b += n_edges * (size_t)p.NF * p.NF * sizeof(__half) + n_edges * sizeof(float);
+        b += n_edges * (size_t)p.NF * precond_ld(p.NF) * sizeof(__half) + n_edges * sizeof(float);
         b += (n_el * Np * Np + 4 * n_el * Np + 2 * B * Np) * sizeof(float);
         b += 3 * p.nt * d;   // M^{-1} x and the two halves of S y
         b += n_edges * P * d;   // tau_hat as FP32 pairs
@@ -1596,7 +1596,7 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
             TRY(dalloc(sim, &S32, nS));
             TRY(dalloc(sim, &aux32, nA));
             TRY(dalloc(sim, &EG32, nE));
-            TRY(dalloc(sim, &sim->Minv16, (size_t)g.n_edges * p.NF * p.NF));
+            TRY(dalloc(sim, &sim->Minv16, (size_t)g.n_edges * p.NF * precond_ld(p.NF)));
             TRY(dalloc(sim, &sim->Mscale, (size_t)g.n_edges));
             TRY(dalloc(sim, &ybuf, p.nt));
             if (!sim->tau32) {

@@ -15,7 +15,7 @@
 //
 // Three launches per product in the refinement residual and the plain product, each short, so
 // that no block waits on a chain of dependent memory round trips:
-//   mf_pre_kernel   y = M^{-1} x, one thread per edge row (block-Jacobi inverse in scaled FP16);
+//   mf_edge_quad_kernel  y = M^{-1} x, four rows a thread (block-Jacobi inverse in scaled FP16);
 //   mf_elem_kernel  one thread per (element, node): the node's traces y gathered straight into
 //                   registers, the operator data loaded before them, the lift, the local solve,
 //                   and the element's half of each face's row -- the edge's minus side (face 1 or
@@ -23,7 +23,7 @@
 //   mf_sum_kernel   y = hm + hp (residual mode: w = g - (hm + hp)), minus half first, so the
 //                   result is the same whatever order the elements ran in.
 // The inner cycles' product is ONE launch: the element pass first forms y = M^{-1} x on each face
-// of its block's elements in shared memory (the same sums as mf_pre_kernel, term for term), and
+// of its block's elements in shared memory, and
 // adds its half of each face's row into the output with a global reduction.  The output is zero
 // beforehand and every row receives at most two addends, so the sum is the same in whichever order
 // the two sides arrive (IEEE addition is commutative) and equals hm + hp of the three-pass form
@@ -74,26 +74,6 @@ constexpr int mf_tile_minb(int t) { return t >= 6 ? 2048 / mf_tile_threads(t) : 
 constexpr int mf_res_threads(int t) { return t == 7 ? 128 : t >= 6 ? 256 : mf_tile_threads(t); }
 constexpr int mf_res_minb(int t) { return t == 6 ? 3 : t == 7 ? 6 : t == 8 ? 4 : 1; }
 
-template <class A>
-__device__ __forceinline__ typename A::T arith_of_f32(float v) {
-    if constexpr (sizeof(typename A::T) == sizeof(float)) return v;
-    else if constexpr (sizeof(typename A::T) == sizeof(float2)) return float2{v, 0.f};
-    else return (double)v;
-}
-
-template <class A, typename TX>
-__device__ __forceinline__ typename A::T arith_load(const TX* p) {
-    if constexpr (sizeof(TX) == sizeof(float)) return arith_of_f32<A>(*p);
-    else return A::from(*p);
-}
-
-// v * 2^k for an arithmetic value (exact: a power of two)
-template <class A>
-__device__ __forceinline__ typename A::T arith_scale(typename A::T v, float s) {
-    if constexpr (std::is_same<typename A::T, float2>::value) return float2{v.x * s, v.y * s};
-    else return v * (typename A::T)s;
-}
-
 // the element's half of a row, stored in the mode's vector type
 template <class A, typename TO>
 __device__ __forceinline__ TO arith_store(typename A::T v) {
@@ -101,85 +81,49 @@ __device__ __forceinline__ TO arith_store(typename A::T v) {
     else return (TO)A::to(v);
 }
 
-// y = M^{-1} x per edge (one thread per row component), y in the arithmetic's own type
-template <int NF, class A, typename TX>
-__device__ __forceinline__ void mf_pre_body(int bid, int n_edges, PrecondBlocks Minv,
-                                            const TX* __restrict__ x, typename A::T* __restrict__ y) {
-    using T = typename A::T;
-    constexpr int EPB = 256 / NF;
-    __shared__ T xs[EPB][NF];
-    const int le = threadIdx.x / NF, ii = threadIdx.x % NF;
-    const int r = bid * EPB + le;
-    const bool live = le < EPB && r < n_edges;
-    if (live) xs[le][ii] = arith_load<A>(x + (size_t)r * NF + ii);
-    __syncthreads();
-    if (!live) return;
-    const __half* M = Minv.h + (size_t)r * NF * NF + ii;
-    typename A::Acc acc;
-#pragma unroll
-    for (int jj = 0; jj < NF; ++jj) acc.add(arith_of_f32<A>(__half2float(M[jj * NF])), xs[le][jj]);
-    y[(size_t)r * NF + ii] = arith_scale<A>(acc.get(), __ldg(Minv.scale + r));
-}
-
-template <int NF, class A, typename TX>
-__global__ void __launch_bounds__(256)
-mf_pre_kernel(int n_edges, PrecondBlocks Minv, const TX* __restrict__ x, typename A::T* __restrict__ y,
-              const int* __restrict__ done) {
-    if (done && *done) return;
-    mf_pre_body<NF, A, TX>(blockIdx.x, n_edges, Minv, x, y);
-}
-
 // y = M^{-1} x on each face (slot le * 4 + f) of the block's elements, into ys -- the sums of
-// mf_pre_body in the same order.  NF % 4 == 0: four rows per thread with 8-byte FP16 loads (x and
-// M^{-1} 16- and 8-byte aligned, checked by the launcher); else one row per thread.
+// mf_quad_body in the same order: four rows per thread with 8-byte FP16 loads; x in 16-byte loads
+// where NF % 4 == 0 (x 16-byte aligned, checked by the launcher).
 template <int P, int EPB>
 __device__ __forceinline__ void mf_face_pre(int bid, const Geom& g, const PrecondBlocks& Minv,
                                             const float* __restrict__ x, float (*ys)[4][3 * P]) {
-    constexpr int NF = 3 * P, NT = EPB * P * P;
-    if constexpr (NF % 4 == 0) {
-        constexpr int Q = NF / 4;
-        for (int u = threadIdx.x; u < EPB * 4 * Q; u += NT) {
-            const int slot = u / Q, q = u % Q, le = slot / 4, f = slot % 4;
-            const int e = bid * EPB + le;
-            if (e >= g.n_el) continue;
-            const int r = edge_of_face(e, f, g);
-            const float4* xr = reinterpret_cast<const float4*>(x + (size_t)r * NF);
-            const __half* M = Minv.h + (size_t)r * NF * NF + 4 * q;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    constexpr int NF = 3 * P, NT = EPB * P * P, LD = precond_ld(NF), Q = LD / 4;
+    for (int u = threadIdx.x; u < EPB * 4 * Q; u += NT) {
+        const int slot = u / Q, q = u % Q, le = slot / 4, f = slot % 4;
+        const int e = bid * EPB + le;
+        if (e >= g.n_el) continue;
+        const int r = edge_of_face(e, f, g);
+        const float* xr = x + (size_t)r * NF;
+        const __half* M = Minv.h + (size_t)r * NF * LD + 4 * q;
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+        float xs[NF];
+        if constexpr (NF % 4 == 0) {
 #pragma unroll
-            for (int jq = 0; jq < Q; ++jq) {
-                const float4 xv = xr[jq];
-                const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const uint2 mv = ld_stream(reinterpret_cast<const uint2*>(M + (size_t)(4 * jq + t) * NF));
-                    const float2 m01 = __half22float2(*reinterpret_cast<const __half2*>(&mv.x));
-                    const float2 m23 = __half22float2(*reinterpret_cast<const __half2*>(&mv.y));
-                    a0 = __fmaf_rn(m01.x, xs[t], a0);
-                    a1 = __fmaf_rn(m01.y, xs[t], a1);
-                    a2 = __fmaf_rn(m23.x, xs[t], a2);
-                    a3 = __fmaf_rn(m23.y, xs[t], a3);
-                }
+            for (int j = 0; j < NF; j += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(xr + j);
+                xs[j] = v.x;
+                xs[j + 1] = v.y;
+                xs[j + 2] = v.z;
+                xs[j + 3] = v.w;
             }
-            const float sc = __ldg(Minv.scale + r);
-            ys[le][f][4 * q] = a0 * sc;
-            ys[le][f][4 * q + 1] = a1 * sc;
-            ys[le][f][4 * q + 2] = a2 * sc;
-            ys[le][f][4 * q + 3] = a3 * sc;
-        }
-    } else {
-        for (int u = threadIdx.x; u < EPB * 4 * NF; u += NT) {
-            const int slot = u / NF, ii = u % NF, le = slot / 4, f = slot % 4;
-            const int e = bid * EPB + le;
-            if (e >= g.n_el) continue;
-            const int r = edge_of_face(e, f, g);
-            const float* xr = x + (size_t)r * NF;
-            const __half* M = Minv.h + (size_t)r * NF * NF + ii;
-            float a = 0.f;
+        } else {
 #pragma unroll
-            for (int jj = 0; jj < NF; ++jj) a = __fmaf_rn(__half2float(M[jj * NF]), xr[jj], a);
-            ys[le][f][ii] = a * __ldg(Minv.scale + r);
+            for (int j = 0; j < NF; ++j) xs[j] = xr[j];
         }
+#pragma unroll
+        for (int j = 0; j < NF; ++j) {
+            const uint2 mv = ld_stream(reinterpret_cast<const uint2*>(M + (size_t)j * LD));
+            const float2 m01 = __half22float2(*reinterpret_cast<const __half2*>(&mv.x));
+            const float2 m23 = __half22float2(*reinterpret_cast<const __half2*>(&mv.y));
+            a[0] = __fmaf_rn(m01.x, xs[j], a[0]);
+            a[1] = __fmaf_rn(m01.y, xs[j], a[1]);
+            a[2] = __fmaf_rn(m23.x, xs[j], a[2]);
+            a[3] = __fmaf_rn(m23.y, xs[j], a[3]);
+        }
+        const float sc = __ldg(Minv.scale + r);
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (NF % 4 == 0 || 4 * q + t < NF) ys[le][f][4 * q + t] = a[t] * sc;
     }
 }
 
@@ -380,57 +324,35 @@ mf_sum_kernel(size_t n, const TO* __restrict__ hm, const TO* __restrict__ hp, co
     }
 }
 
-// qhat = M^{-1} x~ with the FP32 block-Jacobi blocks, FP64-class sums (x split into FP32 pairs).
-template <int NF>
-__device__ __forceinline__ void mf_back_body(int bid, int n_edges, PrecondBlocks Minv,
-                                             const double* __restrict__ x, double* __restrict__ y) {
-    constexpr int EPB = 256 / NF;
-    __shared__ float sxh[EPB][NF], sxl[EPB][NF];
-    const int le = threadIdx.x / NF, ii = threadIdx.x % NF;
-    const int r = bid * EPB + le;
-    const bool live = le < EPB && r < n_edges;
-    if (live) split(x[(size_t)r * NF + ii], sxh[le][ii], sxl[le][ii]);
-    __syncthreads();
-    if (!live) return;
-    const __half* M = Minv.h + (size_t)r * NF * NF;
-    Dot2 acc;
-#pragma unroll
-    for (int jj = 0; jj < NF; ++jj) acc.add(__half2float(M[jj * NF + ii]), 0.f, sxh[le][jj], sxl[le][jj]);
-    const float sc = Minv.scale[r];   // a power of two: scaling the pair is exact
-    y[(size_t)r * NF + ii] = f32_to_f64(acc.p * sc) + f32_to_f64(acc.c * sc);
-}
-
-template <int NF>
-__global__ void __launch_bounds__(256)
-mf_back_kernel(int n_edges, PrecondBlocks Minv, const double* __restrict__ x, double* __restrict__ y) {
-    mf_back_body<NF>(blockIdx.x, n_edges, Minv, x, y);
-}
-
 // The two FP64-class block-Jacobi products -- the refinement residual's y = M^{-1} x as FP32 pairs
-// (PAIRS) and the back-transformation qhat = M^{-1} x~ in FP64 -- with four rows per thread
-// (NF % 4 == 0): the edge's x split into FP32 pairs in shared memory by its threads, then four
-// Dot2 sums over the edge's NF columns from 8-byte FP16 loads.  Each row's sum is mf_pre_body's
-// (ArithF2) or mf_back_body's, term for term.
+// (PAIRS) and the back-transformation qhat = M^{-1} x~ in FP64 -- with four rows per thread: the edge's
+// x split into FP32 pairs in shared memory by its threads, then four Dot2 sums over the edge's NF
+// columns from 8-byte FP16 loads.
+template <int NF>
+__host__ __device__ constexpr int mf_quad_epb() {
+    return 256 / (precond_ld(NF) / 4);
+}
+
 template <int NF, bool PAIRS>
-__global__ void __launch_bounds__(256)
-    mf_edge_quad_kernel(int n_edges, PrecondBlocks Minv, const double* __restrict__ x, void* __restrict__ yv) {
-    static_assert(NF % 4 == 0, "four rows per thread");
-    constexpr int Q = NF / 4, EPB = 256 / Q;
+__device__ __forceinline__ void mf_quad_body(int bid, int n_edges, const PrecondBlocks& Minv,
+                                             const double* __restrict__ x, void* __restrict__ yv) {
+    constexpr int LD = precond_ld(NF), Q = LD / 4, EPB = mf_quad_epb<NF>();
     __shared__ float sxh[EPB][NF], sxl[EPB][NF];
     const int le = threadIdx.x / Q, q = threadIdx.x % Q;
-    const int r = blockIdx.x * EPB + le;
+    const int r = bid * EPB + le;
     const bool live = le < EPB && r < n_edges;
     if (live) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) split(x[(size_t)r * NF + 4 * q + t], sxh[le][4 * q + t], sxl[le][4 * q + t]);
+        for (int t = 0; t < 4; ++t)
+            if (NF % 4 == 0 || 4 * q + t < NF) split(x[(size_t)r * NF + 4 * q + t], sxh[le][4 * q + t], sxl[le][4 * q + t]);
     }
     __syncthreads();
     if (!live) return;
-    const __half* M = Minv.h + (size_t)r * NF * NF + 4 * q;
+    const __half* M = Minv.h + (size_t)r * NF * LD + 4 * q;
     Dot2 acc[4];
 #pragma unroll
     for (int jj = 0; jj < NF; ++jj) {
-        const uint2 mv = ld_stream(reinterpret_cast<const uint2*>(M + jj * NF));
+        const uint2 mv = ld_stream(reinterpret_cast<const uint2*>(M + jj * LD));
         const float2 m01 = __half22float2(*reinterpret_cast<const __half2*>(&mv.x));
         const float2 m23 = __half22float2(*reinterpret_cast<const __half2*>(&mv.y));
         const float xh = sxh[le][jj], xl = sxl[le][jj];
@@ -442,6 +364,7 @@ __global__ void __launch_bounds__(256)
     const float sc = Minv.scale[r];   // a power of two: scaling the pair is exact
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
+        if (NF % 4 != 0 && 4 * q + t >= NF) continue;
         const size_t o = (size_t)r * NF + 4 * q + t;
         if constexpr (PAIRS) {
             float2 pr;
@@ -454,13 +377,20 @@ __global__ void __launch_bounds__(256)
 }
 
 template <int NF, bool PAIRS>
+__global__ void __launch_bounds__(256)
+    mf_edge_quad_kernel(int n_edges, PrecondBlocks Minv, const double* __restrict__ x, void* __restrict__ yv) {
+    mf_quad_body<NF, PAIRS>(blockIdx.x, n_edges, Minv, x, yv);
+}
+
+template <int NF, bool PAIRS>
 void mf_edge_quad_launch(int n_edges, const PrecondBlocks& Minv, const double* x, void* y, cudaStream_t s) {
-    constexpr int EPB = 256 / (NF / 4);
-    mf_edge_quad_kernel<NF, PAIRS><<<(n_edges + EPB - 1) / EPB, EPB * (NF / 4), 0, s>>>(n_edges, Minv, x, y);
+    constexpr int EPB = mf_quad_epb<NF>();
+    mf_edge_quad_kernel<NF, PAIRS>
+        <<<(n_edges + EPB - 1) / EPB, EPB * (precond_ld(NF) / 4), 0, s>>>(n_edges, Minv, x, y);
 }
 
 // Setup: per edge (one block) the FP16 block-Jacobi inverse scaled by the power of two 2^e with
-// max |entry| / 2^e in [0.5, 1), and that scale.
+// max |entry| / 2^e in [0.5, 1), and that scale; columns padded with zeros to precond_ld(NF) rows.
 __global__ void precond_f16_kernel(const double* __restrict__ Minv, int NF, __half* __restrict__ h,
                                    float* __restrict__ scale) {
     const int r = blockIdx.x;
@@ -477,7 +407,11 @@ __global__ void precond_f16_kernel(const double* __restrict__ Minv, int NF, __ha
     int e = 0;
     (void)frexp(red[0], &e);
     if (red[0] == 0.0) e = 0;
-    for (int t = threadIdx.x; t < NF * NF; t += blockDim.x) h[(size_t)r * NF * NF + t] = __double2half(ldexp(M[t], -e));
+    const int LD = precond_ld(NF);
+    for (int t = threadIdx.x; t < NF * LD; t += blockDim.x) {
+        const int c = t / LD, row = t - c * LD;
+        h[(size_t)r * NF * LD + t] = row < NF ? __double2half(ldexp(M[c * NF + row], -e)) : __half(0.f);
+    }
     if (threadIdx.x == 0) scale[r] = ldexpf(1.0f, e);
 }
 
@@ -550,13 +484,11 @@ template <int P, class A, int MODE>
 cudaError_t mf_launch(const Geom& g, const MfOps& op, const void* S, const void* aux, const void* EG, const void* x,
                       const double* rhs, MfVec<MODE>* out, double beta, cudaStream_t s, const int* done,
                       bool out_zeroed = false, double* nrm_scratch = nullptr, double* nrm_out = nullptr) {
-    using T = typename A::T;
     using TO = MfVec<MODE>;
     constexpr int NF = 3 * P;
     if constexpr (MODE == kMfInner) {
-        // the fused pass's vector loads (NF % 4 == 0): x on 16 bytes, the FP16 blocks on 8
-        if (NF % 4 == 0 &&
-            (reinterpret_cast<uintptr_t>(x) % 16 != 0 || reinterpret_cast<uintptr_t>(op.Minv.h) % 8 != 0))
+        // the fused pass's vector loads: the FP16 blocks on 8 bytes, x (NF % 4 == 0) on 16
+        if ((NF % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 != 0) || reinterpret_cast<uintptr_t>(op.Minv.h) % 8 != 0)
             return cudaErrorMisalignedAddress;
         const size_t n = (size_t)g.n_edges * NF;
         if (!out_zeroed) {
@@ -570,13 +502,7 @@ cudaError_t mf_launch(const Geom& g, const MfOps& op, const void* S, const void*
     }
     const void* yv = x;
     if constexpr (MODE != kMfPlain) {
-        if constexpr (MODE == kMfResidual && NF % 4 == 0) {
-            mf_edge_quad_launch<NF, true>(g.n_edges, op.Minv, static_cast<const double*>(x), op.ybuf, s);
-        } else {
-            constexpr int EPE = 256 / NF;
-            mf_pre_kernel<NF, A, TO><<<(g.n_edges + EPE - 1) / EPE, EPE * NF, 0, s>>>(
-                g.n_edges, op.Minv, static_cast<const TO*>(x), static_cast<T*>(op.ybuf), done);
-        }
+        mf_edge_quad_launch<NF, true>(g.n_edges, op.Minv, static_cast<const double*>(x), op.ybuf, s);
         yv = op.ybuf;
     }
     TO* hm = static_cast<TO*>(op.hm);
@@ -600,15 +526,14 @@ cudaError_t mf_launch(const Geom& g, const MfOps& op, const void* S, const void*
 }
 
 // ---- ensembles: the operator's three passes over every group, one persistent launch each -----------
-template <class A, typename TX>
-__global__ void __launch_bounds__(256) ens_mf_pre_kernel(EnsTable t, const TX* __restrict__ x,
-                                                         typename A::T* __restrict__ y, const int* __restrict__ done) {
-    if (done && *done) return;
+template <bool PAIRS>   // y = M^{-1} x: the residual's (FP32 pairs) or the back-transformation (FP64)
+__global__ void __launch_bounds__(256) ens_mf_quad_kernel(EnsTable t, const double* __restrict__ x,
+                                                          double* __restrict__ y) {
     ens_walk(t, [&](const EnsGroup& G, int bid) {
         switch (G.g.P) {
-            case 3: mf_pre_body<9, A, TX>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
-            case 4: mf_pre_body<12, A, TX>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
-            case 5: mf_pre_body<15, A, TX>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
+            case 3: mf_quad_body<9, PAIRS>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
+            case 4: mf_quad_body<12, PAIRS>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
+            case 5: mf_quad_body<15, PAIRS>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
             default: break;
         }
     });
@@ -652,19 +577,8 @@ __global__ void __launch_bounds__(256, MODE == kMfInner ? 6 : 4) ens_mf_elem_ker
     });
 }
 
-__global__ void __launch_bounds__(256) ens_mf_back_kernel(EnsTable t, const double* __restrict__ x, double* __restrict__ y) {
-    ens_walk(t, [&](const EnsGroup& G, int bid) {
-        switch (G.g.P) {
-            case 3: mf_back_body<9>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
-            case 4: mf_back_body<12>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
-            case 5: mf_back_body<15>(bid, G.g.n_edges, G.Minv, x + G.offt, y + G.offt); break;
-            default: break;
-        }
-    });
-}
-
 int ens_edge_blocks(const EnsGroup& G) {
-    const int epb = 256 / (3 * G.g.P);
+    const int epb = 256 / (precond_ld(3 * G.g.P) / 4);   // mf_quad_epb
     return (G.g.n_edges + epb - 1) / epb;
 }
 
@@ -779,10 +693,9 @@ void mf_tile_info(int P, int t, int* epb, int* prefetch) {
 }
 
 cudaError_t launch_ens_mf_inner(const EnsHost& E, const float* x, float* y, cudaStream_t s, const int* done) {
-    // the fused pass's vector loads (3(k + 1) a multiple of 4): x on 16 bytes, the FP16 blocks on 8
+    // the fused pass's vector loads: x on 16 bytes (k = 3), the FP16 blocks on 8
     for (int i = 0; i < E.ngroups; ++i)
-        if ((3 * E.h[i].g.P) % 4 == 0 && (reinterpret_cast<uintptr_t>(x + E.h[i].offt) % 16 != 0 ||
-                                          reinterpret_cast<uintptr_t>(E.h[i].Minv.h) % 8 != 0))
+        if (reinterpret_cast<uintptr_t>(x + E.h[i].offt) % 16 != 0 || reinterpret_cast<uintptr_t>(E.h[i].Minv.h) % 8 != 0)
             return cudaErrorMisalignedAddress;
     const EnsTable tm = ens_table(E, ens_mf_elem_blocks);
     const auto k = ens_mf_elem_kernel<ArithF32, kMfInner>;
@@ -794,12 +707,13 @@ cudaError_t launch_ens_mf_inner(const EnsHost& E, const float* x, float* y, cuda
 cudaError_t launch_ens_mf_residual(const EnsHost& E, const MfOps& scratch, size_t nt, const double* x,
                                    const double* rhs, double* w, cudaStream_t s) {
     const EnsTable te = ens_table(E, ens_edge_blocks), tm = ens_table(E, ens_mf_elem_blocks);
-    float2* y = static_cast<float2*>(scratch.ybuf);
+    double* y = static_cast<double*>(scratch.ybuf);   // (FP32 pairs)
     double *hm = static_cast<double*>(scratch.hm), *hp = static_cast<double*>(scratch.hp);
-    const auto kp = ens_mf_pre_kernel<ArithF2, double>;
+    const auto kp = ens_mf_quad_kernel<true>;
     const auto ke = ens_mf_elem_kernel<ArithF2, kMfResidual>;
-    kp<<<ens_grid(kp, te.start[te.ngroups]), 256, 0, s>>>(te, x, y, nullptr);
-    ke<<<ens_grid(ke, tm.start[tm.ngroups]), 256, 0, s>>>(tm, nullptr, y, hm, hp, nullptr);
+    kp<<<ens_grid(kp, te.start[te.ngroups]), 256, 0, s>>>(te, x, y);
+    ke<<<ens_grid(ke, tm.start[tm.ngroups]), 256, 0, s>>>(tm, nullptr, reinterpret_cast<const float2*>(y), hm, hp,
+                                                                      nullptr);
     mf_sum_kernel<double, true><<<sum_grid(nt), 256, 0, s>>>(nt, hm, hp, rhs, w, nullptr);
     count_launches(3);
     return cudaGetLastError();
@@ -807,7 +721,8 @@ cudaError_t launch_ens_mf_residual(const EnsHost& E, const MfOps& scratch, size_
 
 cudaError_t launch_ens_mf_back(const EnsHost& E, const double* x, double* y, cudaStream_t s) {
     const EnsTable te = ens_table(E, ens_edge_blocks);
-    ens_mf_back_kernel<<<ens_grid(ens_mf_back_kernel, te.start[te.ngroups]), 256, 0, s>>>(te, x, y);
+    const auto k = ens_mf_quad_kernel<false>;
+    k<<<ens_grid(k, te.start[te.ngroups]), 256, 0, s>>>(te, x, y);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -815,9 +730,7 @@ cudaError_t launch_ens_mf_back(const EnsHost& E, const double* x, double* y, cud
 cudaError_t launch_mf_back(const Geom& g, const PrecondBlocks& Minv, const double* x, double* y, cudaStream_t s) {
 #define CASE(P, NF)                                                                                      \
     case P: {                                                                                            \
-        constexpr int EPB = 256 / NF;                                                                    \
-        if constexpr (NF % 4 == 0) mf_edge_quad_launch<NF, false>(g.n_edges, Minv, x, y, s);             \
-        else mf_back_kernel<NF><<<(g.n_edges + EPB - 1) / EPB, EPB * NF, 0, s>>>(g.n_edges, Minv, x, y); \
+        mf_edge_quad_launch<NF, false>(g.n_edges, Minv, x, y, s);                                        \
         count_launches(1);                                                                               \
         return cudaGetLastError();                                                                       \
     }
