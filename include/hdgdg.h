@@ -232,7 +232,7 @@ enum {
     HDGDG_KT_CONDENSE = 2,  /* A^{-1} R1 and the trace right-hand side */
     HDGDG_KT_RECOVER = 3,   /* local recovery of Q and L_i */
     HDGDG_KT_DG = 4,        /* DG residual of the nonlinear part */
-    HDGDG_KT_COMBINE = 5,   /* stage combinations and the final update */
+    HDGDG_KT_COMBINE = 5,   /* stage combinations and the final update (explicit stages form theirs in HDGDG_KT_DG) */
     HDGDG_KT_RESIDUAL = 6,  /* end of each restart cycle: the correction x += V y, the true residual
                                g - S x and its norm */
     HDGDG_KT_GUESS = 7,     /* initial guess of each trace solve: candidate residual norms, the

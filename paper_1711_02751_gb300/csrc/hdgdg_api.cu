@@ -1313,55 +1313,63 @@ hdgdg_status one_step_graph(hdgdg_sim* sim) {
     return HDGDG_OK;
 }
 
-// Explicit SSP Runge-Kutta on the whole DG residual (the paper's RK2 DG / RK3 DG), with the
+// n explicit SSP Runge-Kutta steps on the whole DG residual (the paper's RK2 DG / RK3 DG), with the
 // stage increments K_i = dt M^{-1} R(q_i):
 //   RK2 (Heun):        q1 = q + K1;                 q' = q + K1/2 + K2/2
 //   RK3 (Shu-Osher):   q1 = q + K1;  q2 = q + K1/4 + K2/4;  q' = q + K1/6 + K2/6 + 2 K3/3
-hdgdg_status explicit_step(hdgdg_sim* sim) {
-    NvtxRange nv("time_step");
-    const size_t n3 = 3 * sim->plan.n;
+// The steps are queued one behind the other and the host waits once: a step that produces a
+// non-finite value sets the flag that makes every later launch write nothing, so the state is left at
+// the last finite step, and the device's count says which that is.
+hdgdg_status explicit_steps(hdgdg_sim* sim, int n) {
+    NvtxRange nv("time_steps");
     cudaStream_t st = sim->stream;
     const double dt = sim->cfg.dt;
-    auto rhs = [&](const double* qi, double* K, double ti) -> hdgdg_status {
-        TimedGroup tg(sim, HDGDG_KT_DG);
-        CU(launch_dg_full(sim->g, qi, sim->phiB, dt, sim->fface, K, st, ti));
-        return HDGDG_OK;
-    };
-    const double t0 = sim->t;
-    auto comb = [&](double* out, std::initializer_list<std::pair<double*, double>> terms, unsigned* flag) -> hdgdg_status {
-        CombineTerms t{};
-        for (auto& pr : terms) { t.X[t.n] = pr.first; t.c[t.n++] = pr.second; }
-        TimedGroup tg(sim, HDGDG_KT_COMBINE);
-        CU(launch_combine(n3, sim->q, t, out, flag, st));
-        return HDGDG_OK;
-    };
+    unsigned* const bad = sim->flags;
+    unsigned* const begun = sim->flags + 1;
+    double* buf[2] = {sim->q, sim->q_new};
     double *K1 = sim->NLs[0], *K2 = sim->NLs[1], *K3 = sim->NLs[2];
-    TRY(rhs(sim->q, K1, t0));
-    TRY(comb(sim->Qs, {{K1, 1.0}}, nullptr));
-    TRY(rhs(sim->Qs, K2, t0 + dt));
-    CU(cudaMemsetAsync(sim->flags, 0, sizeof(unsigned), st));
-    if (sim->cfg.scheme == HDGDG_RK2) {
-        TRY(comb(sim->q_new, {{K1, 0.5}, {K2, 0.5}}, sim->flags));
-    } else {
-        TRY(comb(sim->R1, {{K1, 0.25}, {K2, 0.25}}, nullptr));
-        TRY(rhs(sim->R1, K3, t0 + 0.5 * dt));
-        TRY(comb(sim->q_new, {{K1, 1.0 / 6.0}, {K2, 1.0 / 6.0}, {K3, 2.0 / 3.0}}, sim->flags));
+    CU(cudaMemsetAsync(sim->flags, 0, 2 * sizeof(unsigned), st));
+    double t = sim->t;
+    for (int k = 0; k < n; ++k, t += dt) {
+        const double* q = buf[k & 1];
+        auto stage = [&](const double* qi, double ti, std::initializer_list<std::pair<double*, double>> terms, double* to,
+                         bool first, bool last) -> hdgdg_status {
+            FinalSource f;   // this stage's increment is the last term
+            f.base = q;
+            for (auto& pr : terms) { f.t.X[f.t.n] = pr.first; f.t.c[f.t.n++] = pr.second; }
+            f.slot = f.t.n - 1;
+            f.qn = to;
+            f.guard = bad;
+            if (last) f.nonfinite = bad;
+            else f.out = const_cast<double*>(f.t.X[f.slot]);
+            TimedGroup tg(sim, HDGDG_KT_DG);
+            CU(launch_dg_full_stage(sim->g, qi, sim->phiB, dt, sim->fface, f, first ? begun : nullptr, st, ti));
+            return HDGDG_OK;
+        };
+        double* next = buf[(k + 1) & 1];
+        TRY(stage(q, t, {{K1, 1.0}}, sim->Qs, true, false));
+        if (sim->cfg.scheme == HDGDG_RK2) {
+            TRY(stage(sim->Qs, t + dt, {{K1, 0.5}, {K2, 0.5}}, next, false, true));
+        } else {
+            TRY(stage(sim->Qs, t + dt, {{K1, 0.25}, {K2, 0.25}}, sim->R1, false, false));
+            TRY(stage(sim->R1, t + 0.5 * dt, {{K1, 1.0 / 6.0}, {K2, 1.0 / 6.0}, {K3, 2.0 / 3.0}}, next, false, true));
+        }
     }
-    unsigned flag = 0;
-    CU(cudaMemcpyAsync(&sim->hbuf[0], sim->flags, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    unsigned flag[2] = {0, 0};
+    CU(cudaMemcpyAsync(&sim->hbuf[0], sim->flags, sizeof(flag), cudaMemcpyDeviceToHost, st));
     TRY(sync(sim));
-    std::memcpy(&flag, &sim->hbuf[0], sizeof(unsigned));
-    if (flag) return fail(sim, HDGDG_ENONFINITE, "step %lld produced a non-finite state", sim->stats.steps + 1);
-    std::swap(sim->q, sim->q_new);
-    sim->stats.steps += 1;
-    sim->t += dt;
+    std::memcpy(flag, &sim->hbuf[0], sizeof(flag));
+    const int done = flag[0] ? (int)flag[1] - 1 : n;
+    for (int k = 0; k < done; ++k) sim->t += dt;
+    sim->stats.steps += done;
+    if (done & 1) std::swap(sim->q, sim->q_new);
+    if (flag[0]) return fail(sim, HDGDG_ENONFINITE, "step %lld produced a non-finite state", sim->stats.steps + 1);
     return HDGDG_OK;
 }
 
 hdgdg_status one_step(hdgdg_sim* sim) {
     if (use_step_graph(sim)) return one_step_graph(sim);
     NvtxRange nv("time_step");
-    if (explicit_scheme(&sim->cfg)) return explicit_step(sim);
     const size_t n3 = 3 * sim->plan.n;
     cudaStream_t st = sim->stream;
     for (int i = 0; i < sim->s; ++i) {
@@ -1867,9 +1875,11 @@ hdgdg_status hdgdg_step(hdgdg_sim* sim, int n_steps) {
     if (!sim) return HDGDG_EINVAL;
     if (n_steps < 0) return fail(sim, HDGDG_EINVAL, "n_steps < 0");
     if (!sim->have_state) return fail(sim, HDGDG_ESTATE, "step before set_state");
-    for (int k = 0; k < n_steps; ++k) {
+    constexpr int kQueued = 64;   // explicit steps queued before the host waits
+    const bool queued = explicit_scheme(&sim->cfg);
+    for (int k = 0; k < n_steps; k += queued ? kQueued : 1) {
         const long long l0 = launches_total();
-        const hdgdg_status st = one_step(sim);
+        const hdgdg_status st = queued ? explicit_steps(sim, std::min(kQueued, n_steps - k)) : one_step(sim);
         sim->stats.kernel_launches += launches_total() - l0;
         if (st != HDGDG_OK) return st;
     }

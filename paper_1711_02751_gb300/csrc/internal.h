@@ -226,21 +226,26 @@ cudaError_t launch_dg_nl_f32(const Geom& g, const double* q, const double* phiB,
 // the same residual with its inputs (state, phi_B, tau) rounded to BF16 and FP32 arithmetic (k <= 4)
 cudaError_t launch_dg_nl_bf16(const Geom& g, const double* q, const double* phiB, const double* tau_edge,
                               double scale, double* fface, double* out, cudaStream_t s, double t = 0.0);
-// out = scale * M^{-1} (the explicit DG residual of the whole flux with the source term)
-cudaError_t launch_dg_full(const Geom& g, const double* q, const double* phiB, double scale,
-                           double* fface, double* out, cudaStream_t s, double t = 0.0);
+// One stage of an explicit scheme: K = scale M^{-1} (the DG residual of the whole flux with the source
+// term) into fin.out (kept when not null) and fin.qn = base + sum_k t.c[k] t.X[k] with K as term
+// `slot`, as launch_combine forms it.  Steps may be queued one behind the other: where *fin.guard is set
+// nothing is written, and `count` (the first stage's) counts the steps begun without it.
+cudaError_t launch_dg_full_stage(const Geom& g, const double* q, const double* phiB, double scale, double* fface,
+                                 const FinalSource& fin, unsigned* count, cudaStream_t s, double t);
 
 struct CombineTerms {
     const double* X[10];
     double c[10];
     int n;
 };
-struct FinalSource {   // launch_dg_nl_f32io's final update
+struct FinalSource {   // an update formed by the element pass: launch_dg_nl_f32io, launch_dg_full_stage
     const double* base = nullptr;
     CombineTerms t{};
     int slot = -1;
     double* qn = nullptr;
     unsigned* nonfinite = nullptr;
+    double* out = nullptr;            // the residual itself (explicit stages)
+    const unsigned* guard = nullptr;  // set: write nothing
 };
 // out = base + sum_t c_t X_t over n doubles (out may alias base)
 cudaError_t launch_combine(size_t n, const double* base, const CombineTerms& t, double* out,

@@ -152,10 +152,26 @@ dg_face_kernel(Geom g, const TQ* __restrict__ q, const std::conditional_t<A32, f
     dg_face_body<P, FULL, Tc, BF, TQ, A32>(blockIdx.x, g, q, phiB, tau_edge, fface, t_bc);
 }
 
+// The face pass of an explicit stage (launch_dg_full_stage)
+template <int P>
+__global__ void __launch_bounds__(256)
+dg_face_stage_kernel(Geom g, const double* __restrict__ q, const double* __restrict__ phiB, double* __restrict__ fface,
+                     double t_bc, const unsigned* __restrict__ guard, unsigned* count) {
+    if (*guard) return;
+    if (count && blockIdx.x == 0 && threadIdx.x == 0) *count += 1u;
+    dg_face_body<P, true, double>(blockIdx.x, g, q, phiB, nullptr, fface, t_bc);
+}
+
 // The step's final update at node o (field stride fs) with this pass's residual v as term
 // fin.slot: every other term's loads issued before the sums, each field's terms added in their
 // order as combine_kernel adds them.
 __device__ __forceinline__ void dg_final_update(const FinalSource& fin, size_t o, size_t fs, const double v[3]) {
+    if (fin.guard && *(const volatile unsigned*)fin.guard) return;   // (past the pass's barriers)
+    if (fin.out) {
+        fin.out[o] = v[0];
+        fin.out[o + fs] = v[1];
+        fin.out[o + 2 * fs] = v[2];
+    }
     double acc[3], x[kFinalTerms][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[c] = fin.base[o + c * fs];
@@ -408,6 +424,22 @@ cudaError_t dg_launch(const Geom& g, const double* q, const double* phiB, const 
     return cudaGetLastError();
 }
 
+// An explicit stage: the face pass, and the element pass that also forms the stage's update.  As two
+// passes, a separate combination and a host wait a step, RK2 on 20^2, k = 8 took 78 us a step, 42 of
+// them in kernels (FP64 pipe: 12 us an element pass of 32 400 nodes, 6.4 a face pass); as queued
+// stages of two launches 53.
+template <int P>
+cudaError_t dg_stage_launch(const Geom& g, const double* q, const double* phiB, double scale, double* fface,
+                            const FinalSource& fin, unsigned* count, cudaStream_t s, double t) {
+    constexpr int EPB = DgTile<P>::EPB;
+    const int nf = g.n_edges * P;
+    dg_face_stage_kernel<P><<<(nf + 255) / 256, 256, 0, s>>>(g, q, phiB, fface, t, fin.guard, count);
+    dg_volume_kernel<P, true, double, false, double, false, true>
+        <<<(g.n_el + EPB - 1) / EPB, EPB * P * P, 0, s>>>(g, q, phiB, fface, scale, nullptr, fin);
+    count_launches(2);
+    return cudaGetLastError();
+}
+
 // The mixed form's residual on FP32 copies: phi_B, tau and the face fluxes in FP32, the state
 // in FP32 (q32, the recovery's FP32 stage values) or FP64 (q64, the step's start).
 template <int P>
@@ -549,17 +581,15 @@ cudaError_t launch_dg_nl_bf16(const Geom& g, const double* q, const double* phiB
     }
 }
 
-cudaError_t launch_dg_full(const Geom& g, const double* q, const double* phiB, double scale,
-                           double* fface, double* out, cudaStream_t s, double t) {
+cudaError_t launch_dg_full_stage(const Geom& g, const double* q, const double* phiB, double scale, double* fface,
+                                 const FinalSource& fin, unsigned* count, cudaStream_t s, double t) {
+    if (!fin.base || !fin.qn || !fin.guard || fin.t.n < 1 || fin.t.n > kFinalTerms || fin.slot < 0 || fin.slot >= fin.t.n)
+        return cudaErrorInvalidValue;
     switch (g.P) {
-        case 2: return dg_launch<2, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 3: return dg_launch<3, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 4: return dg_launch<4, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 5: return dg_launch<5, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 6: return dg_launch<6, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 7: return dg_launch<7, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 8: return dg_launch<8, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
-        case 9: return dg_launch<9, true>(g, q, phiB, nullptr, scale, fface, out, s, t);
+#define CASE(P) \
+    case P: return dg_stage_launch<P>(g, q, phiB, scale, fface, fin, count, s, t);
+        CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8) CASE(9)
+#undef CASE
         default: return cudaErrorInvalidValue;
     }
 }
