@@ -26,7 +26,28 @@ namespace {
 template <int P>
 struct DgTile {
     static constexpr int Np = P * P;
-    static constexpr int EPB = (256 / Np) > 0 ? (256 / Np) : 1;   // elements per block
+    static constexpr int EPB = (256 / Np) > 0 ? (256 / Np) : 1;   // elements per block, at most
+};
+
+// Both passes of a mesh with work for less than every SM's blocks of 256 threads take smaller blocks, so
+// that it reaches more SMs: an FP64 warp instruction holds its SM quarter for ~60 cycles, and the
+// eight warps of a full block queue for four pipes while other SMs idle.  Blocks of
+// 64 edge nodes and of one element for each SM's share: RK2 on 20^2, k = 8 53 -> 50 us a step, ARS2 on 8^2,
+// k = 2 2 % less a step; from 152 full blocks on the full ones stay (the same grid as before).
+constexpr int kSms = 152;
+template <int P>
+struct DgGrid {
+    int ft, fgrid;   // face pass: threads a block (one per edge node), blocks
+    int vt, vgrid;   // element pass: threads a block (whole elements), blocks
+    explicit DgGrid(const Geom& g) {
+        const int nf = g.n_edges * P;
+        ft = nf <= kSms * 256 ? 64 : 256;
+        fgrid = (nf + ft - 1) / ft;
+        int epb = (g.n_el + kSms - 1) / kSms;
+        if (epb > DgTile<P>::EPB) epb = DgTile<P>::EPB;
+        vt = epb * P * P;
+        vgrid = (g.n_el + epb - 1) / epb;
+    }
 };
 
 // An input of the residual in the arithmetic type; BF: rounded to BF16 first (8 significant bits,
@@ -79,7 +100,7 @@ __device__ __forceinline__ void dg_face_body(int bid, const Geom& g, const TQ* _
                                              double t_bc) {
     using TV = std::conditional_t<A32, float, double>;   // the node values as the pass holds them
     constexpr int Np = P * P;
-    const int t = bid * 256 + threadIdx.x;
+    const int t = bid * (int)blockDim.x + threadIdx.x;
     if (t >= g.n_edges * P) return;
     const int r = t / P, b = t % P;
     int em, fm, ep, fp;
@@ -144,12 +165,12 @@ __device__ __forceinline__ void dg_face_body(int bid, const Geom& g, const TQ* _
     }
 }
 
-template <int P, bool FULL, typename Tc, bool BF = false, typename TQ = double, bool A32 = false>
+template <int P, typename Tc, bool BF = false, typename TQ = double, bool A32 = false>
 __global__ void __launch_bounds__(256)
 dg_face_kernel(Geom g, const TQ* __restrict__ q, const std::conditional_t<A32, float, double>* __restrict__ phiB,
                const std::conditional_t<A32, float, double>* __restrict__ tau_edge,
                std::conditional_t<A32, float, double>* __restrict__ fface, double t_bc) {
-    dg_face_body<P, FULL, Tc, BF, TQ, A32>(blockIdx.x, g, q, phiB, tau_edge, fface, t_bc);
+    dg_face_body<P, false, Tc, BF, TQ, A32>(blockIdx.x, g, q, phiB, tau_edge, fface, t_bc);
 }
 
 // The face pass of an explicit stage (launch_dg_full_stage)
@@ -217,8 +238,9 @@ __device__ __forceinline__ void dg_volume_body(int bid, const Geom& g, const TQ*
 
     const int le = threadIdx.x / Np;
     const int n = threadIdx.x % Np;
-    const int e = bid * EPB + le;
-    const bool live = le < EPB && e < g.n_el;
+    const int epb = (int)blockDim.x / Np;   // elements of this block (<= EPB; threads past them idle)
+    const int e = bid * epb + le;
+    const bool live = le < epb && e < g.n_el;
     const size_t fs = (size_t)g.n_el * Np;
     const int i = n % P, j = n / P;
 
@@ -411,31 +433,27 @@ __global__ void mass_final_kernel(const double* partial, int nb, double J, doubl
     if (threadIdx.x == 0) *out = J * acc;
 }
 
-template <int P, bool FULL, typename Tc = double, bool BF = false>
+template <int P, typename Tc = double, bool BF = false>
 cudaError_t dg_launch(const Geom& g, const double* q, const double* phiB, const double* tau_edge,
                       double scale, double* fface, double* out, cudaStream_t s, double t) {
-    constexpr int EPB = DgTile<P>::EPB;
-    const int nf = g.n_edges * P;
-    dg_face_kernel<P, FULL, Tc, BF><<<(nf + 255) / 256, 256, 0, s>>>(g, q, phiB, tau_edge, fface, t);
-    count_launches(1);
-    dg_volume_kernel<P, FULL, Tc, BF><<<(g.n_el + EPB - 1) / EPB, EPB * P * P, 0, s>>>(g, q, phiB, fface, scale, out,
-                                                                                      FinalSource{});
-    count_launches(1);
+    const DgGrid<P> d(g);
+    dg_face_kernel<P, Tc, BF><<<d.fgrid, d.ft, 0, s>>>(g, q, phiB, tau_edge, fface, t);
+    dg_volume_kernel<P, false, Tc, BF><<<d.vgrid, d.vt, 0, s>>>(g, q, phiB, fface, scale, out, FinalSource{});
+    count_launches(2);
     return cudaGetLastError();
 }
 
 // An explicit stage: the face pass, and the element pass that also forms the stage's update.  As two
 // passes, a separate combination and a host wait a step, RK2 on 20^2, k = 8 took 78 us a step, 42 of
 // them in kernels (FP64 pipe: 12 us an element pass of 32 400 nodes, 6.4 a face pass); as queued
-// stages of two launches 53.
+// stages of two launches 53, with the smaller blocks of DgGrid 50.
 template <int P>
 cudaError_t dg_stage_launch(const Geom& g, const double* q, const double* phiB, double scale, double* fface,
                             const FinalSource& fin, unsigned* count, cudaStream_t s, double t) {
-    constexpr int EPB = DgTile<P>::EPB;
-    const int nf = g.n_edges * P;
-    dg_face_stage_kernel<P><<<(nf + 255) / 256, 256, 0, s>>>(g, q, phiB, fface, t, fin.guard, count);
+    const DgGrid<P> d(g);
+    dg_face_stage_kernel<P><<<d.fgrid, d.ft, 0, s>>>(g, q, phiB, fface, t, fin.guard, count);
     dg_volume_kernel<P, true, double, false, double, false, true>
-        <<<(g.n_el + EPB - 1) / EPB, EPB * P * P, 0, s>>>(g, q, phiB, fface, scale, nullptr, fin);
+        <<<d.vgrid, d.vt, 0, s>>>(g, q, phiB, fface, scale, nullptr, fin);
     count_launches(2);
     return cudaGetLastError();
 }
@@ -446,20 +464,18 @@ template <int P>
 cudaError_t dg_launch_f32io(const Geom& g, const double* q64, const float* q32, const float* phiB,
                             const float* tau_edge, double scale, float* fface, double* out, cudaStream_t s,
                             double t, const FinalSource& fin) {
-    constexpr int EPB = DgTile<P>::EPB;
-    const int nf = g.n_edges * P;
-    const int gf = (nf + 255) / 256, gv = (g.n_el + EPB - 1) / EPB, tv = EPB * P * P;
+    const DgGrid<P> d(g);
     if (q32) {
-        dg_face_kernel<P, false, float, false, float, true><<<gf, 256, 0, s>>>(g, q32, phiB, tau_edge, fface, t);
+        dg_face_kernel<P, float, false, float, true><<<d.fgrid, d.ft, 0, s>>>(g, q32, phiB, tau_edge, fface, t);
         if (fin.base)
-            dg_volume_kernel<P, false, float, false, float, true, true><<<gv, tv, 0, s>>>(g, q32, phiB, fface, scale,
+            dg_volume_kernel<P, false, float, false, float, true, true><<<d.vgrid, d.vt, 0, s>>>(g, q32, phiB, fface, scale,
                                                                                         out, fin);
         else
-            dg_volume_kernel<P, false, float, false, float, true><<<gv, tv, 0, s>>>(g, q32, phiB, fface, scale, out,
+            dg_volume_kernel<P, false, float, false, float, true><<<d.vgrid, d.vt, 0, s>>>(g, q32, phiB, fface, scale, out,
                                                                                   fin);
     } else {
-        dg_face_kernel<P, false, float, false, double, true><<<gf, 256, 0, s>>>(g, q64, phiB, tau_edge, fface, t);
-        dg_volume_kernel<P, false, float, false, double, true><<<gv, tv, 0, s>>>(g, q64, phiB, fface, scale, out,
+        dg_face_kernel<P, float, false, double, true><<<d.fgrid, d.ft, 0, s>>>(g, q64, phiB, tau_edge, fface, t);
+        dg_volume_kernel<P, false, float, false, double, true><<<d.vgrid, d.vt, 0, s>>>(g, q64, phiB, fface, scale, out,
                                                                                  fin);
     }
     count_launches(2);
@@ -526,14 +542,14 @@ void count_launches(int n) { g_launches.fetch_add(n); }
 cudaError_t launch_dg_nl(const Geom& g, const double* q, const double* phiB, const double* tau_edge,
                          double scale, double* fface, double* out, cudaStream_t s, double t) {
     switch (g.P) {
-        case 2: return dg_launch<2, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 3: return dg_launch<3, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 4: return dg_launch<4, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 5: return dg_launch<5, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 6: return dg_launch<6, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 7: return dg_launch<7, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 8: return dg_launch<8, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 9: return dg_launch<9, false>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 2: return dg_launch<2>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 3: return dg_launch<3>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 4: return dg_launch<4>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 5: return dg_launch<5>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 6: return dg_launch<6>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 7: return dg_launch<7>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 8: return dg_launch<8>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 9: return dg_launch<9>(g, q, phiB, tau_edge, scale, fface, out, s, t);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -558,14 +574,14 @@ cudaError_t launch_dg_nl_f32io(const Geom& g, const double* q64, const float* q3
 cudaError_t launch_dg_nl_f32(const Geom& g, const double* q, const double* phiB, const double* tau_edge,
                              double scale, double* fface, double* out, cudaStream_t s, double t) {
     switch (g.P) {
-        case 2: return dg_launch<2, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 3: return dg_launch<3, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 4: return dg_launch<4, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 5: return dg_launch<5, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 6: return dg_launch<6, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 7: return dg_launch<7, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 8: return dg_launch<8, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 9: return dg_launch<9, false, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 2: return dg_launch<2, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 3: return dg_launch<3, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 4: return dg_launch<4, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 5: return dg_launch<5, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 6: return dg_launch<6, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 7: return dg_launch<7, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 8: return dg_launch<8, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 9: return dg_launch<9, float>(g, q, phiB, tau_edge, scale, fface, out, s, t);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -573,10 +589,10 @@ cudaError_t launch_dg_nl_f32(const Geom& g, const double* q, const double* phiB,
 cudaError_t launch_dg_nl_bf16(const Geom& g, const double* q, const double* phiB, const double* tau_edge,
                               double scale, double* fface, double* out, cudaStream_t s, double t) {
     switch (g.P) {
-        case 2: return dg_launch<2, false, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 3: return dg_launch<3, false, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 4: return dg_launch<4, false, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
-        case 5: return dg_launch<5, false, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 2: return dg_launch<2, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 3: return dg_launch<3, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 4: return dg_launch<4, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
+        case 5: return dg_launch<5, float, true>(g, q, phiB, tau_edge, scale, fface, out, s, t);
         default: return cudaErrorInvalidValue;
     }
 }
