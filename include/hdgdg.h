@@ -140,7 +140,8 @@ typedef struct {
                             thread per row component, neighbour vectors gathered through shared
                             memory; 1 = a persistent kernel that also streams the matrix through
                             shared memory with bulk (TMA) copies, two stages deep.  Identical
-                            results (same summation order). */
+                            results (same summation order).  Solves that run as one launch
+                            (host_steps) carry a product of their own: no effect there. */
     int krylov_ortho;    /* Gram-Schmidt of the mixed form's FP32 inner cycles: 0 = classical,
                             applied twice (CGS2; with the matrix-free operator the second pass
                             is delayed into the next Arnoldi step, whose product is taken of the
@@ -175,6 +176,9 @@ typedef struct {
                             buffers (a handful of them, cached per handle) and replayed: the choice of
                             each trace solve's start, its restart cycles (a conditional while node)
                             and their stop tests run on the device, and the host waits once per step.
+                            On the assembled matrix a system whose Krylov basis fits the device's
+                            shared memory is solved by one cooperative launch instead (also in
+                            host-driven steps).  Explicit schemes queue their steps, 64 per host wait.
                             1: host-driven steps (the host waits for each restart cycle).  Steps run
                             host-driven anyway while the kernel-class timers are on and for
                             prescribed time-dependent boundary traces (HDGDG_VORTEX).  Same results
@@ -227,7 +231,8 @@ typedef struct {
 
 /* Kernel classes of the per-kernel timers (hdgdg_kernel_time). */
 enum {
-    HDGDG_KT_SPMV = 0,      /* trace-matrix product of the Krylov loop (one kernel per launch) */
+    HDGDG_KT_SPMV = 0,      /* trace-matrix product of the Krylov loop (one kernel per launch; a solve
+                               in one launch: its parts' times by the device clock) */
     HDGDG_KT_ORTHO = 1,     /* Gram-Schmidt dots, updates and normalisation of one iteration */
     HDGDG_KT_CONDENSE = 2,  /* A^{-1} R1 and the trace right-hand side */
     HDGDG_KT_RECOVER = 3,   /* local recovery of Q and L_i */
