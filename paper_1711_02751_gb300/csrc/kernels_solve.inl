@@ -1032,7 +1032,13 @@ __global__ void __launch_bounds__(kNT, 1) solve_kernel(const __grid_constant__ S
 template <int NF, typename T>
 cudaError_t solve_launch(const SolveArgs& a, cudaStream_t s) {
     const void* f = reinterpret_cast<const void*>(solve_kernel<NF, T>);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.plan.smem);
+    // the kernel's limit is set to the device's, the same in every call: handles of different sizes share
+    // it from several threads, between one's setting and its launch (or its graph's instantiation)
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)sizeof(Shared) - 64);
     if (e != cudaSuccess) return e;
     SolveArgs arg = a;
     void* params[] = {&arg};

@@ -64,3 +64,25 @@ def test_streamed_product_past_the_one_launch_size():
             outs.append(s.get_state())
     for p, q in zip(*outs):
         assert np.array_equal(p, q)
+
+
+def test_handles_of_different_sizes_in_threads():
+    """Handles of one degree and different shared-memory needs created and stepped from eight threads:
+    every step succeeds and gives the lone run's state bit for bit."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    def run(N):
+        nn = (N * N, 9)
+        x, y = hd.node_coords(N, 2)
+        h = 1.0 + 0.01 * np.sin(2 * np.pi * x) * np.cos(2 * np.pi * y)
+        with hd.Sim(N, 2, 0.2 / N, np.zeros(nn), **MIXED) as s:
+            s.set_state(h, np.zeros(nn), np.zeros(nn))
+            s.step(3)
+            return np.concatenate([np.ravel(f) for f in s.get_state()])
+
+    sizes = [4, 24, 48, 64]
+    lone = {N: run(N) for N in sizes}
+    order = sizes * 16
+    with ThreadPoolExecutor(8) as pool:
+        for N, got in zip(order, pool.map(run, order)):
+            assert np.array_equal(got, lone[N])
