@@ -359,6 +359,13 @@ hdgdg_status hdgdg_set_local_tiles(hdgdg_sim* sim, int condense_tile, int recove
 hdgdg_status hdgdg_stage_solve(hdgdg_sim* sim, const double* R1, double* Q, double* qhat,
                                int* iterations);
 
+/* Failure detection of the trace solves that run as one launch (host_steps): its blocks wait for one
+ * another, each wait for at most `loads` loads (0 = the default, 2^22 trips to the L2 cache, a few
+ * seconds); where one runs out the launch ends and the step or stage solve returns ECUDA.  lost = 1
+ * (tests): one contribution to the next exchange is taken back, so that its waits run out.  EINVAL
+ * for a handle whose solves are not one launch. */
+hdgdg_status hdgdg_set_solve_wait(hdgdg_sim* sim, unsigned loads, int lost);
+
 /* ---- measurement helpers --------------------------------------------------------- */
 
 /* Switch the per-kernel-class timers on (1) or off (0) and zero them.  When on, the

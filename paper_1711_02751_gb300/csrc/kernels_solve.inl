@@ -43,7 +43,6 @@ namespace {
 constexpr int kNT = kSolveThreads, kNW = kNT / 32;
 constexpr int kCtlWarps = 2;                    // warps 0 and 1: Hessenberg column, rotation, stop test
 constexpr int kProdThreads = kNT - 32 * kCtlWarps;
-constexpr unsigned kMaxSpins = 1u << 22;        // bound of every wait
 
 // Values that cross blocks: each 32-bit half in an 8-byte word (accessed at once) under the 32-bit
 // number of the exchange it belongs to.
@@ -180,16 +179,21 @@ struct Solver {
         sh.last = now;
     }
 
-    // Whether to stop waiting after `spins` fruitless loads (each a trip to L2, so kMaxSpins are one to
-    // two seconds): the error word is then set, and every later wait of every block ends early.
+    // Whether to stop waiting after `spins` fruitless loads: the error word is then set, and every later
+    // wait of every block ends early.
     __device__ __forceinline__ bool give_up(unsigned spins) {
         if ((spins & 63u) != 63u) return false;
-        if (*(volatile int*)&sh.gave_up == 0 && *reinterpret_cast<volatile int*>(a.error) == 0 && spins < kMaxSpins)
+        if (*(volatile int*)&sh.gave_up == 0 && *reinterpret_cast<volatile int*>(a.error) == 0 && spins < a.max_spins)
             return false;
         atomicExch(a.error, 3);
         *(volatile int*)&sh.gave_up = 1;
         return true;
     }
+
+    // A block barrier, and whether a wait of this block has run out: one answer for every thread.  (Read
+    // after the barrier, the flag may already be set by a thread that has gone on to its next wait; the
+    // threads that saw it would leave, and the others wait for them at a barrier without end.)
+    __device__ __forceinline__ bool any_gave_up() { return __syncthreads_or(*(volatile int*)&sh.gave_up) != 0; }
 
     __device__ __forceinline__ u64* a_buffer() {
         return a.A + (size_t)abuf * a.n_edges * NF * Tagged<T>::kWords;
@@ -314,8 +318,7 @@ struct Solver {
                 if (outp) outp[c] = s;
             }
         }
-        __syncthreads();
-        return sh.gave_up == 0;
+        return !any_gave_up();
     }
 
     // The neighbour traces of ng own edge rows from g0 on, of the vector published in `buf` by the
@@ -789,9 +792,9 @@ struct Solver {
             const int tid = thread_index();
             if (tid >= 32 * kCtlWarps) product(tid - 32 * kCtlWarps, a_buffer(), tag, V + j * ld);
             else if (j > 0) control(j - 1);
-            __syncthreads();
+            const bool out = any_gave_up();
             mark(0);
-            if (sh.gave_up) return -1;
+            if (out) return -1;
             if (j > 0 && sh.done) return j;
             contribute<T, true>(V, ld, j + 1, z, false, R);
             if (!collect<T>(j + 1, sh.h1, h1t)) return -1;
@@ -835,9 +838,9 @@ struct Solver {
             const int tid = thread_index();
             if (tid >= 32 * kCtlWarps) product(tid - 32 * kCtlWarps, a_buffer(), tag, ao);
             else if (j > 0) control(j - 1);
-            __syncthreads();
+            const bool out = any_gave_up();
             mark(0);
-            if (sh.gave_up) return -1;
+            if (out) return -1;
             if (j > 0 && sh.done) return j;
             if (j == 0) {
                 for (int r = tid; r < R; r += kNT) {

@@ -1,0 +1,48 @@
+"""A wait of the one-launch trace solve that runs out (a contribution that never comes, the wait bounded
+to a few milliseconds): the launch ends by itself, the call returns ECUDA and the device stays usable."""
+import numpy as np
+import pytest
+
+from paper_1711_02751_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+hd = pytest.importorskip("paper_1711_02751_gb300.hdgdg")
+
+LOADS = 4096
+FORMS = {"fp64": {}, "mixed": dict(precision="mixed", local_precision="f32x2", residual_f32x2=True)}
+
+
+def _state(N, k):
+    x, y = hd.node_coords(N, k)
+    h, hu, hv, b = W.large_state(x, y, seed=7)
+    return h, hu, hv, b, W.advective_dt(x, h, hu, hv, N)
+
+
+@pytest.mark.parametrize("host_steps", [False, True])
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_a_lost_contribution_ends_the_step_with_an_error(form, host_steps):
+    h, hu, hv, b, dt = _state(24, 3)
+    with hd.Sim(24, 3, dt, bottom=b, host_steps=host_steps, **FORMS[form]) as s:
+        s.set_state(h, hu, hv)
+        s.step(2)
+        before = s.get_state()
+        s.set_solve_wait(LOADS, lost=True)
+        with pytest.raises(hd.HdgdgError) as ex:
+            s.step(1)
+        assert ex.value.status == hd.ECUDA and "wait" in str(ex.value)
+        assert s.stats()["steps"] == 2
+        for a, c in zip(before, s.get_state()):
+            assert np.array_equal(a, c)
+    with hd.Sim(24, 3, dt, bottom=b, host_steps=host_steps, **FORMS[form]) as s:
+        s.set_state(h, hu, hv)
+        s.step(2)
+        for a, c in zip(before, s.get_state()):
+            assert np.array_equal(a, c)
+
+
+def test_only_one_launch_solves_have_such_waits():
+    h, hu, hv, b, dt = _state(8, 2)
+    with hd.Sim(8, 2, dt, bottom=b, precision="mixed", local_precision="f32x2", trace_operator=1) as s:
+        with pytest.raises(hd.HdgdgError) as ex:
+            s.set_solve_wait(LOADS)
+        assert ex.value.status == hd.EINVAL
