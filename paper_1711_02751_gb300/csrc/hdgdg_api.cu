@@ -908,6 +908,28 @@ cudaError_t dg_nl_enqueue(hdgdg_sim* sim, const double* Qi, bool stage_value, do
     return launch_dg_nl(sim->g, Qi, sim->phiB, sim->tau, sim->cfg.dt, sim->fface, out, st, t);
 }
 
+// The state that the one-launch solves of a handle keep between launches, as before the first: no
+// value may carry an exchange's number by chance.  (A and X lie in the global basis' bytes.)
+cudaError_t reset_exchange(hdgdg_sim* sim, cudaStream_t st) {
+    const bool f32 = sim->cfg.precision == HDGDG_MIXED;
+    void* const basis = f32 ? static_cast<void*>(sim->V32) : sim->V;
+    cudaError_t e = cudaMemsetAsync(sim->solve_part, 0, solve_part_bytes(kSolveMaxBlocks), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sim->solve_epoch, 0, 32 * sizeof(unsigned), st);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(basis, 0, basis_vectors(&sim->cfg) * sim->plan.nt * (f32 ? sizeof(float) : sizeof(double)), st);
+    return e;
+}
+
+// A bounded wait of the trace solve ran out (the stream has been waited for): the blocks left at
+// different exchanges, whose numbers and words the next launch would otherwise meet again, and some may
+// have stored their part of a solution.  The handle goes on from the last completed step, without history.
+hdgdg_status solve_wait_ran_out(hdgdg_sim* sim, unsigned flag) {
+    for (int i = 0; i < sim->s; ++i) sim->n_hist[i] = 0;
+    if (sim->splan.on) CU(reset_exchange(sim, sim->stream));
+    CU(cudaMemsetAsync(spmv_error(sim), 0, sizeof(int), sim->stream));
+    return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag);
+}
+
 // ---- the trace solve as one launch ----------------------------------------------------------------
 // The whole solve of gmres_solve -- start, restart cycles, back-transformation, history store --
 // enqueued on st as one cooperative launch (kernels_solve.inl); its counters are added to sstats.
@@ -983,7 +1005,7 @@ hdgdg_status solve_one_launch(hdgdg_sim* sim, const double* g, double* qhat, int
     StepStats ss;
     std::memcpy(flag, sim->hbuf, sizeof(flag));
     std::memcpy(&ss, sim->hbuf + 4, sizeof(ss));
-    if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
+    if (flag[3]) return solve_wait_ran_out(sim, flag[3]);
     if (eb) {   // the launch's time, divided among the kernel classes as its first block's clock saw them
         SolveClocks ck;
         std::memcpy(&ck, sim->hbuf + 16, sizeof(ck));
@@ -1297,7 +1319,7 @@ hdgdg_status one_step_graph(hdgdg_sim* sim) {
     if (bad) {   // the history slots may hold this step's partial solves: start the next solves afresh
         for (int i = 0; i < sim->s; ++i) sim->n_hist[i] = 0;
         if (flag[2]) return fail(sim, HDGDG_ECUDA, "a bounded wait of a local kernel ran out (%u)", flag[2]);
-        if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
+        if (flag[3]) return solve_wait_ran_out(sim, flag[3]);
         if (ss.nonfinite) return fail(sim, HDGDG_ENONFINITE, "non-finite trace right-hand side or GMRES residual");
         if (ss.notconv) {
             sim->stats.last_krylov_iterations = ss.notconv_its;
@@ -1416,7 +1438,7 @@ hdgdg_status one_step(hdgdg_sim* sim) {
     TRY(sync(sim));
     std::memcpy(flag, &sim->hbuf[0], sizeof(flag));
     if (flag[2]) return fail(sim, HDGDG_ECUDA, "a bounded wait of a local kernel ran out (%u)", flag[2]);
-    if (flag[3]) return fail(sim, HDGDG_ECUDA, "a bounded wait of the trace solve ran out (%u)", flag[3]);
+    if (flag[3]) return solve_wait_ran_out(sim, flag[3]);
     if (flag[0]) return fail(sim, HDGDG_ENONFINITE, "step %lld produced a non-finite state", sim->stats.steps + 1);
     std::swap(sim->q, sim->q_new);
     sim->stats.steps += 1;
@@ -1519,12 +1541,7 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
         sim->splan = plan_solve(g.n_edges, g.P, p.m, c->precision == HDGDG_MIXED);
         TRY(dalloc(sim, &sim->solve_part, solve_part_bytes(kSolveMaxBlocks) / sizeof(*sim->solve_part)));
         TRY(dalloc(sim, &sim->solve_epoch, 32));
-        // no value may carry an exchange's number by chance
-        CU(cudaMemsetAsync(sim->solve_part, 0, solve_part_bytes(kSolveMaxBlocks), sim->stream));
-        CU(cudaMemsetAsync(sim->solve_epoch, 0, 32 * sizeof(unsigned), sim->stream));
-        const bool f32 = c->precision == HDGDG_MIXED;
-        void* basis = f32 ? static_cast<void*>(sim->V32) : sim->V;
-        CU(cudaMemsetAsync(basis, 0, basis_vectors(c) * p.nt * (f32 ? sizeof(float) : sizeof(double)), sim->stream));
+        CU(reset_exchange(sim, sim->stream));
     }
     if (!c->host_steps) {
         CU(cudaStreamCreateWithFlags(&sim->body_stream, cudaStreamNonBlocking));

@@ -46,3 +46,34 @@ def test_only_one_launch_solves_have_such_waits():
         with pytest.raises(hd.HdgdgError) as ex:
             s.set_solve_wait(LOADS)
         assert ex.value.status == hd.EINVAL
+
+
+@pytest.mark.parametrize("host_steps", [False, True])
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_the_handle_goes_on_after_a_lost_contribution(form, host_steps):
+    """The exchange's numbers and words start afresh: the steps after the failed one are those of a handle
+    that lost nothing, bit for bit, again and again, and so is a stage solve."""
+    h, hu, hv, b, dt = _state(24, 3)
+    with hd.Sim(24, 3, dt, bottom=b, host_steps=host_steps, **FORMS[form]) as s, \
+            hd.Sim(24, 3, dt, bottom=b, host_steps=host_steps, **FORMS[form]) as ref:
+        s.set_state(h, hu, hv)
+        s.step(3)
+        for steps, scale in ((1, 1.0), (6, 0.5)):
+            for sim in (s, ref):
+                sim.set_state(h, scale * hu, scale * hv)
+            s.set_solve_wait(LOADS, lost=True)
+            with pytest.raises(hd.HdgdgError) as ex:
+                s.step(1)
+            assert ex.value.status == hd.ECUDA
+            s.set_solve_wait()
+            s.step(steps)
+            ref.step(steps)
+            for a, c in zip(ref.get_state(), s.get_state()):
+                assert np.array_equal(a, c)
+        R1 = np.random.default_rng(3).standard_normal((3, 24 * 24, 16))
+        want = ref.stage_solve(R1)[1]
+        s.set_solve_wait(LOADS, lost=True)
+        with pytest.raises(hd.HdgdgError):
+            s.stage_solve(R1)
+        s.set_solve_wait()
+        assert np.array_equal(s.stage_solve(R1)[1], want)
