@@ -141,7 +141,8 @@ typedef struct {
                             memory; 1 = a persistent kernel that also streams the matrix through
                             shared memory with bulk (TMA) copies, two stages deep.  Identical
                             results (same summation order).  Solves that run as one launch
-                            (host_steps) carry a product of their own: no effect there. */
+                            (host_steps) carry a product of their own: no effect there, unless
+                            hdgdg_set_solve_blocks(sim, 0) keeps a launch per operation. */
     int krylov_ortho;    /* Gram-Schmidt of the mixed form's FP32 inner cycles: 0 = classical,
                             applied twice (CGS2; with the matrix-free operator the second pass
                             is delayed into the next Arnoldi step, whose product is taken of the
@@ -178,7 +179,7 @@ typedef struct {
                             and their stop tests run on the device, and the host waits once per step.
                             On the assembled matrix a system whose Krylov basis fits the device's
                             shared memory is solved by one cooperative launch instead (also in
-                            host-driven steps).  Explicit schemes queue their steps, 64 per host wait.
+                            host-driven steps; hdgdg_set_solve_blocks).  Explicit schemes queue their steps, 64 per host wait.
                             1: host-driven steps (the host waits for each restart cycle).  Steps run
                             host-driven anyway while the kernel-class timers are on and for
                             prescribed time-dependent boundary traces (HDGDG_VORTEX).  Same results
@@ -358,6 +359,14 @@ hdgdg_status hdgdg_set_local_tiles(hdgdg_sim* sim, int condense_tile, int recove
  * (may be NULL).  *iterations (may be NULL) receives the GMRES iteration count. */
 hdgdg_status hdgdg_stage_solve(hdgdg_sim* sim, const double* R1, double* Q, double* qhat,
                                int* iterations);
+
+/* Blocks of the trace solves that run as one launch (host_steps): < 0 = one an SM (create's choice),
+ * 0 = a launch per operation instead, n > 0 = at most n blocks, and a launch per operation where the
+ * system does not fit them.  For handles that share the device: a solve over every SM keeps the other
+ * handles' kernels waiting for as long as it runs.  Chosen before the first step, never by load, since
+ * a grid has its own order of sums: results agree to the solver tolerance, not bit for bit.  No effect on handles whose
+ * solves are not one launch. */
+hdgdg_status hdgdg_set_solve_blocks(hdgdg_sim* sim, int blocks);
 
 /* Failure detection of the trace solves that run as one launch (host_steps): its blocks wait for one
  * another, each wait for at most `loads` loads (0 = the default, 2^22 trips to the L2 cache, a few

@@ -357,7 +357,7 @@ struct hdgdg_sim {
     GmresCtl* ctl = nullptr;
     CycleGraph cycle_graph[4];   // [FP64 form, mixed form] x [timers off, on]
     // the trace solve as one cooperative launch (small and mid-size systems on the assembled matrix)
-    SolvePlan splan;
+    SolvePlan splan, splan_create;     // as it runs now, and as laid out at create (one block an SM)
     unsigned long long* solve_part = nullptr;
     unsigned* solve_epoch = nullptr;   // then the count, and at 16 words the launch's SolveClocks
     unsigned solve_spins = kSolveMaxSpins;   // bound of its waits
@@ -1538,7 +1538,7 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
     CU(cudaMallocHost(&sim->hhist, kMaxStages * sizeof(DevHist)));
     TRY(dalloc(sim, &sim->dls, kLsSlots));
     if (!matrix_free(c)) {
-        sim->splan = plan_solve(g.n_edges, g.P, p.m, c->precision == HDGDG_MIXED);
+        sim->splan = sim->splan_create = plan_solve(g.n_edges, g.P, p.m, c->precision == HDGDG_MIXED);
         TRY(dalloc(sim, &sim->solve_part, solve_part_bytes(kSolveMaxBlocks) / sizeof(*sim->solve_part)));
         TRY(dalloc(sim, &sim->solve_epoch, 32));
         CU(reset_exchange(sim, sim->stream));
@@ -2127,6 +2127,20 @@ hdgdg_status hdgdg_stage_solve(hdgdg_sim* sim, const double* R1, double* Q, doub
     if (iterations) *iterations = its;
     TRY(download(sim, Q, sim->Qs, n3));
     if (qhat) TRY(download(sim, qhat, sim->lam, sim->plan.nt));
+    return HDGDG_OK;
+}
+
+hdgdg_status hdgdg_set_solve_blocks(hdgdg_sim* sim, int blocks) {
+    if (!sim) return HDGDG_EINVAL;
+    SolvePlan p = sim->splan_create;
+    if (p.on && blocks == 0) p.on = false;
+    else if (p.on && blocks > 0)
+        p = plan_solve(sim->g.n_edges, sim->g.P, sim->plan.m, sim->cfg.precision == HDGDG_MIXED, blocks);
+    if (p.on == sim->splan.on && p.blocks == sim->splan.blocks) return HDGDG_OK;
+    CU(cudaStreamSynchronize(sim->stream));
+    drop_step_graphs(sim);
+    if (p.on) CU(reset_exchange(sim, sim->stream));   // (the basis of the other path may lie there)
+    sim->splan = p;
     return HDGDG_OK;
 }
 

@@ -7,7 +7,7 @@ namespace hdgdg {
 
 cudaError_t launch_solve_f64(int P, const SolveArgs& a, cudaStream_t s) { return solve_dispatch<double>(P, a, s); }
 
-SolvePlan plan_solve(int n_edges, int P, int m, bool fp32) {
+SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks) {
     SolvePlan p;
     int dev = 0, sms = 0, coop = 0, smem_max = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -19,6 +19,7 @@ SolvePlan plan_solve(int n_edges, int P, int m, bool fp32) {
     }
     if (!coop || sms < 1) return p;
     sms = std::min(sms, kSolveMaxBlocks);
+    if (max_blocks > 0) sms = std::min(sms, max_blocks);
     const int NF = 3 * P;
     const size_t t = fp32 ? 4 : 8;
     // at least kMinRows rows a block: below that an exchange grows faster than the work shrinks; FP32

@@ -83,8 +83,9 @@ inline size_t solve_part_bytes(int blocks) { return 2 * (size_t)kSolveMaxCols * 
 // global memory, which the one-launch solve keeps in shared memory.
 constexpr int solve_basis_vectors(bool fp32) { return fp32 ? 8 : 6; }
 // The layout for a system of n_edges edge rows of degree P - 1, restart length m, FP64 or FP32
-// cycles; on = false where it does not fit the device's shared memory.
-SolvePlan plan_solve(int n_edges, int P, int m, bool fp32);
+// cycles, over at most max_blocks blocks (0: one an SM); on = false where it does not fit their shared
+// memory.
+SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks = 0);
 cudaError_t launch_solve_f64(int P, const SolveArgs& a, cudaStream_t s);
 cudaError_t launch_solve_f32(int P, const SolveArgs& a, cudaStream_t s);
 
