@@ -72,10 +72,21 @@ bool explicit_scheme(const hdgdg_config* c) { return c->scheme == HDGDG_RK2 || c
 
 int restart_of(const hdgdg_config* c) { return c->krylov_restart > 0 ? c->krylov_restart : 10; }
 
+size_t edge_rows(const hdgdg_config* c) {
+    const size_t N = (size_t)c->n_side, B = c->batch > 0 ? (size_t)c->batch : 1;
+    return B * (c->boundary != HDGDG_PERIODIC ? 2 * N * (N + 1) : 2 * N * N);
+}
+
+// whether the handle has room for trace solves in one launch (of a larger system: none is held)
+bool solve_room(const hdgdg_config* c) {
+    return !matrix_free(c) && !explicit_scheme(c) && edge_rows(c) <= (size_t)1 << 30 &&
+           solve_fits((int)edge_rows(c), c->degree_k + 1, restart_of(c), c->precision == HDGDG_MIXED);
+}
+
 // Krylov basis vectors in global memory (at least what the one-launch solve keeps there instead)
 size_t basis_vectors(const hdgdg_config* c) {
     const int m1 = restart_of(c) + 1;
-    return (size_t)(matrix_free(c) ? m1 : std::max(m1, solve_basis_vectors(c->precision == HDGDG_MIXED)));
+    return (size_t)(solve_room(c) ? std::max(m1, solve_basis_vectors(c->precision == HDGDG_MIXED)) : m1);
 }
 
 // order of the trace-solve initial guess (0: start from zero)
@@ -91,7 +102,7 @@ Plan make_plan(const hdgdg_config* c) {
     const size_t N = (size_t)c->n_side, P = (size_t)c->degree_k + 1;
     const size_t B = c->batch > 0 ? (size_t)c->batch : 1;
     const size_t n_el = B * N * N, Np = P * P;
-    const size_t n_edges = B * (c->boundary != HDGDG_PERIODIC ? 2 * N * (N + 1) : 2 * N * N);
+    const size_t n_edges = edge_rows(c);
     p.n = n_el * Np;
     p.NV = (int)(3 * Np);
     p.NF = (int)(3 * P);
@@ -124,7 +135,7 @@ Plan make_plan(const hdgdg_config* c) {
     }
     b += (reduction_scratch_doubles(p.m, (int)n_edges, (int)P) + mass_scratch_doubles() + 4 * (size_t)(p.m + 2) + 16) * d;
     b += 64 + sizeof(GmresCtl);                               // flags, GMRES control block
-    if (!matrix_free(c)) b += solve_part_bytes(kSolveMaxBlocks) + 128;  // the one-launch solve's exchanges
+    if (solve_room(c)) b += solve_part_bytes(kSolveMaxBlocks) + 128;    // the one-launch solve's exchanges
     if (c->local_precision == HDGDG_LOCAL_FP32) b += n_el * (size_t)p.NV * p.NV * sizeof(float);
     if (c->local_precision == HDGDG_LOCAL_BF16) b += tc_image_bytes((int)P);
     if (c->local_precision == HDGDG_LOCAL_BF16_SPLIT) b += tc_split_image_bytes((int)P);
@@ -1537,7 +1548,7 @@ hdgdg_status setup(hdgdg_sim* sim, const double* bottom_b) {
     TRY(dalloc(sim, &sim->dhist, kMaxStages));
     CU(cudaMallocHost(&sim->hhist, kMaxStages * sizeof(DevHist)));
     TRY(dalloc(sim, &sim->dls, kLsSlots));
-    if (!matrix_free(c)) {
+    if (solve_room(c)) {
         sim->splan = sim->splan_create = plan_solve(g.n_edges, g.P, p.m, c->precision == HDGDG_MIXED);
         TRY(dalloc(sim, &sim->solve_part, solve_part_bytes(kSolveMaxBlocks) / sizeof(*sim->solve_part)));
         TRY(dalloc(sim, &sim->solve_epoch, 32));

@@ -7,19 +7,11 @@ namespace hdgdg {
 
 cudaError_t launch_solve_f64(int P, const SolveArgs& a, cudaStream_t s) { return solve_dispatch<double>(P, a, s); }
 
-SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks) {
+namespace {
+
+// The layout over at most sms blocks of smem_max bytes of shared memory
+SolvePlan lay_out(int n_edges, int P, int m, bool fp32, int sms, int smem_max) {
     SolvePlan p;
-    int dev = 0, sms = 0, coop = 0, smem_max = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return p;
-    }
-    if (!coop || sms < 1) return p;
-    sms = std::min(sms, kSolveMaxBlocks);
-    if (max_blocks > 0) sms = std::min(sms, max_blocks);
     const int NF = 3 * P;
     const size_t t = fp32 ? 4 : 8;
     // at least kMinRows rows a block: below that an exchange grows faster than the work shrinks; FP32
@@ -42,5 +34,24 @@ SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks) {
     p.on = true;
     return p;
 }
+
+}  // namespace
+
+SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks) {
+    int dev = 0, sms = 0, coop = 0, smem_max = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return SolvePlan{};
+    }
+    if (!coop || sms < 1) return SolvePlan{};
+    sms = std::min(sms, kSolveMaxBlocks);
+    if (max_blocks > 0) sms = std::min(sms, max_blocks);
+    return lay_out(n_edges, P, m, fp32, sms, smem_max);
+}
+
+bool solve_fits(int n_edges, int P, int m, bool fp32) { return lay_out(n_edges, P, m, fp32, 152, 227 * 1024).on; }
 
 }  // namespace hdgdg

@@ -86,6 +86,9 @@ constexpr int solve_basis_vectors(bool fp32) { return fp32 ? 8 : 6; }
 // cycles, over at most max_blocks blocks (0: one an SM); on = false where it does not fit their shared
 // memory.
 SolvePlan plan_solve(int n_edges, int P, int m, bool fp32, int max_blocks = 0);
+// Whether the system fits one launch on GB300 (152 SMs, 227 KB of shared memory a block): what a handle has
+// room for.  No device call.
+bool solve_fits(int n_edges, int P, int m, bool fp32);
 cudaError_t launch_solve_f64(int P, const SolveArgs& a, cudaStream_t s);
 cudaError_t launch_solve_f32(int P, const SolveArgs& a, cudaStream_t s);
 
