@@ -241,13 +241,11 @@ struct Solver {
                         for (int r = sg * rs + (lane & 7); r < hi; r += 8) s = add(s, __fmul_rn(p[r], zz[r]));
                     }
                 } else {
-                    U acc = U(0);
 #pragma unroll 4
                     for (int r = sg * rs + (lane & 7); r < hi; r += 8) {
-                        if constexpr (DOT) acc += p[r] * zz[r];
-                        else acc += p[r];
+                        if constexpr (DOT) s += p[r] * zz[r];
+                        else s = add(s, p[r]);
                     }
-                    s = SumOf<U>::of(acc);
                 }
             }
             s = add(s, shfl_xor(s, 4));
@@ -597,19 +595,19 @@ struct Solver {
         contribute<double, false>(sq, 0, 1, nullptr, false, R);
     }
 
-    // ||g||^2 and the squared residual norms of the start's candidates (guess_norms_body and, FP32
-    // cycles, guess_norms_x2_body term for term): the exchange begun
+    // ||g||^2 and the squared residual norms of the start's candidates (the terms of guess_norms_body or, FP32
+    // cycles, guess_norms_x2_body; those added as FP32 pairs from the first on): the exchange begun
     __device__ __forceinline__ void candidates(int avail) {
         const int tid = thread_index();
         if (kF32 && avail > 0) {
-            float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            PairSum acc[7] = {};
             for (int r = tid; r < R; r += kNT) {
                 const double gv = a.g[r0 + r], y0 = a.dh->y[0][r0 + r];
                 const float gh = f64_to_f32(gv), e = f64_to_f32(gv - y0);
                 float d[6];
 #pragma unroll
                 for (int j = 1; j < 6; ++j) d[j] = j < avail ? f64_to_f32(y0 - a.dh->y[j][r0 + r]) : 0.f;
-                acc[0] = __fmaf_rn(gh, gh, acc[0]);
+                acc[0] = add(acc[0], __fmul_rn(gh, gh));
 #pragma unroll
                 for (int q = 1; q < 7; ++q) {
                     if (q > avail) break;
@@ -617,13 +615,13 @@ struct Solver {
 #pragma unroll
                     for (int j = 1; j < 6; ++j)
                         if (j < q) v = __fmaf_rn(f64_to_f32(a.coef[q][j]), d[j], v);
-                    acc[q] = __fmaf_rn(v, v, acc[q]);
+                    acc[q] = add(acc[q], __fmul_rn(v, v));
                 }
             }
-            float* buf = reinterpret_cast<float*>(V);
+            PairSum* buf = reinterpret_cast<PairSum*>(V);
 #pragma unroll
             for (int q = 0; q < 7; ++q) buf[q * kGuessLd + tid] = acc[q];
-            contribute<float, false>(buf, kGuessLd, avail + 1, nullptr, false, min(R, kNT));
+            contribute<PairSum, false>(buf, kGuessLd, avail + 1, nullptr, false, min(R, kNT));
         } else {
             double acc[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
             for (int r = tid; r < R; r += kNT) {

@@ -1,6 +1,11 @@
 // Sums across lanes, warps and blocks: FP64, or for FP32 terms FP32 pairs (hi + lo with |lo| <= ulp(hi) / 2,
 // about 48 bits; TwoSum), which keeps reductions of FP32 kernels off GB300's FP64 pipe -- one FP64 warp
-// instruction holds an SM partition's pipe for about 60 cycles.
+// instruction holds an SM partition's pipe for about 60 cycles.  Against exact sums, pairs and FP64 sums
+// of the same FP32 terms (dots, nearly orthogonal dots and norms of 18 432 to 400 000 unit-scaled random
+// values) are off by the same 4.74e-10 to 9.0e-11, equal to six digits: the terms' own rounding.
+// FP64 sums instead, from the lanes to the exchange: 32^2, k = 2 5.96 -> 7.06 ms over ten steps, 91^2, k = 3
+// 9.85 -> 11.1, 16 x 32^2, k = 3 28.8 -> 30.9; as 64-bit integers 6.5, 10.3 and 29.7; states the same bit
+// for bit but one (4e-15 apart).
 #pragma once
 
 #include "compensated.h"
@@ -34,12 +39,14 @@ __device__ __forceinline__ double value(double v) { return v; }
 template <typename T>   // double
 struct SumOf {
     using S = double;
-    static __device__ __forceinline__ S of(T v) { return v; }
 };
 template <>
 struct SumOf<float> {
     using S = PairSum;
-    static __device__ __forceinline__ S of(float v) { return PairSum{v, 0.f}; }
+};
+template <>
+struct SumOf<PairSum> {
+    using S = PairSum;
 };
 
 }  // namespace hdgdg
