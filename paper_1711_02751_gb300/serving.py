@@ -28,6 +28,14 @@ import numpy as np
 from . import hdgdg as hd
 from . import workloads as W
 
+# Blocks of each request's one-launch trace solves: a fixed share of the SMs, whatever else runs, so that
+# results do not depend on the mix.  A solve over every SM keeps the other requests' kernels waiting: a
+# 256 x 256, k = 4 handle beside seven of 32 x 32 to 128 x 128 took 75 ms a step (7.9 alone; 14.5 beside
+# solves of 32 blocks, 12.8 beside a launch per operation).  40 requests at 4/s, time to solution p50 / p99 in s at
+# 16, 24, 32, 48, 64 and 152 blocks: 4.1 / 6.7, 4.7 / 7.8, 3.3 / 6.5, 3.2 / 6.3, 3.2 / 6.4, 5.4 / 9.4; 256
+# instances in batches: 4.8e8, -, 4.9e8, -, 4.4e8 and 4.4e8 DOF-steps/s.
+SOLVE_BLOCKS = 32
+
 
 @dataclass
 class Request:
@@ -138,6 +146,7 @@ def run_batch(batch, chunk=10):
     n = batch.N * batch.N
     with hd.Sim(batch.N, batch.k, float(dts.max()), bottom=cat(3), batch=len(states), dt_per_instance=dts,
                 **form_options(batch.precision)) as s:
+        s.set_solve_blocks(SOLVE_BLOCKS)
         s.set_state(cat(0), cat(1), cat(2))
         done = 0
         while done < batch.steps:
@@ -162,6 +171,7 @@ def run_one(req, chunk=10):
     """Run one request to completion on a fresh handle; returns the final (h, hu, hv)."""
     h, hu, hv, b, dt = initial_state(req)
     with hd.Sim(req.N, req.k, dt, bottom=b, **form_options(req.precision)) as s:
+        s.set_solve_blocks(SOLVE_BLOCKS)
         s.set_state(h, hu, hv)
         done = 0
         while done < req.steps:
