@@ -551,6 +551,9 @@ double beta_of(const hdgdg_sim* sim) { return sim->cfg.dt * sim->a_ii * sim->g.t
 // A restart cycle that cannot halve a true residual already below kStagnation * ||g|| has reached
 // the rounding floor of the FP64 residual: the solve accepts it.
 constexpr double kStagnationFloor = 1e-12;
+// A cycle stops once it has reduced its starting residual this much: FP32 cycles 1e6 times, FP64 ones by
+// the solve's tolerance alone.
+constexpr double inner_reduction(bool fp32) { return fp32 ? 1e-6 : 0.0; }
 // Extrapolation coefficients of the initial guess, order q = 1..6: x_0 = sum_j c[q][j] x_{n-1-j}.
 constexpr double kGuessCoef[7][6] = {{0, 0, 0, 0, 0, 0},     {1, 0, 0, 0, 0, 0},     {2, -1, 0, 0, 0, 0},
                                      {3, -3, 1, 0, 0, 0},    {4, -6, 4, -1, 0, 0},   {5, -10, 10, -5, 1, 0},
@@ -682,8 +685,7 @@ hdgdg_status gmres_solve(hdgdg_sim* sim, const double* g, double* qhat, int* ite
     const size_t n = sim->plan.nt;
     const double rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
     const int maxit = sim->cfg.krylov_maxit > 0 ? sim->cfg.krylov_maxit : 2000;
-    // Mixed form: an FP32 cycle stops once it has reduced its starting residual 1e6 times.
-    const double inner_rel = kMixed ? 1e-6 : 0.0;
+    const double inner_rel = inner_reduction(kMixed);
     constexpr double kStagnation = kStagnationFloor;
     cudaStream_t st = sim->stream;
     GmresCtl* ctl = sim->ctl;
@@ -977,6 +979,7 @@ cudaError_t solve_enqueue_one_launch(hdgdg_sim* sim, const double* g, double* qh
     a.dh = dh;
     std::memcpy(a.coef, kGuessCoef, sizeof(kGuessCoef));
     a.rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
+    a.inner_rel = inner_reduction(kMixed);
     a.maxit = sim->cfg.krylov_maxit > 0 ? sim->cfg.krylov_maxit : 2000;
     a.stagnation = kStagnationFloor;
     a.sc = sim->sctl;
@@ -986,7 +989,7 @@ cudaError_t solve_enqueue_one_launch(hdgdg_sim* sim, const double* g, double* qh
         cudaError_t e = launch_multidot(g, 0, 1, g, n, sim->red, sim->dls + 32, st, &dh->has_history);
         if (e == cudaSuccess) e = launch_guess_gram_dev(n, g, dh, sim->red, sim->dls, st);
         if (e == cudaSuccess)
-            e = launch_ls_start_dev(n, g, dh, sim->dls, a.rtol, 1e-6, a.maxit, sim->ctl, sim->sctl, sim->sstats,
+            e = launch_ls_start_dev(n, g, dh, sim->dls, a.rtol, a.inner_rel, a.maxit, sim->ctl, sim->sctl, sim->sstats,
                                     dv_nrm(sim), sim->xt, sim->w, st);
         if (e != cudaSuccess) return e;
         a.start_given = true;
@@ -1065,7 +1068,7 @@ cudaError_t solve_enqueue_graph(hdgdg_sim* sim, const double* g, double* qhat, i
     const size_t n = sim->plan.nt;
     const double rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
     const int maxit = sim->cfg.krylov_maxit > 0 ? sim->cfg.krylov_maxit : 2000;
-    const double inner_rel = kMixed ? 1e-6 : 0.0;
+    const double inner_rel = inner_reduction(kMixed);
     const int order = guess_order(&sim->cfg);
     const bool history = stage >= 0 && order > 0;
     if (sim->splan.on) return solve_enqueue_one_launch<T>(sim, g, qhat, history ? sim->dhist + stage : nullptr, nullptr, st);

@@ -972,7 +972,7 @@ struct Solver {
             if (tid == 0) {
                 sh.s[0] = rn;
                 sh.done = 0;
-                sh.tol_cycle = fmax(sh.tol, (kF32 ? 1e-6 : 0.0) * rn);
+                sh.tol_cycle = fmax(sh.tol, a.inner_rel * rn);
             }
             __syncthreads();
             const int cols = spent ? 0 : cycle(rn);
