@@ -12,7 +12,8 @@
 // FP64 cycles delay the second pass: w1 is published and its product corrected to that of v through
 // A V = V H (launch_dcgs_fused), which hides the publication behind an exchange.  FP32 cycles keep
 // the order of the launch-per-operation path in every FP32 sum that a solution depends on -- products,
-// dots, updates: where a solve ends within its tolerance depends on their rounding.
+// updates, and the dots' groups of four (see contribute): where a solve ends within its tolerance
+// depends on their rounding.
 // A restart cycle adds two exchanges' worth of waiting (x~ published; the true residual's norm).
 // Every block sums all blocks' partial sums itself, in block order, and takes every decision from
 // the same numbers.  There is no fenced barrier: every value that crosses blocks -- partial sums,
@@ -207,9 +208,11 @@ struct Solver {
     // nv columns cols + c * ldc (times zz when DOT).  Groups of eight lanes take one column each, the
     // four groups of a warp adjacent columns of the same rows; the rows are cut into segments so that
     // every warp has work.  FP32 dots add the products of four consecutive rows (aligned to four in the
-    // whole vector; single products when its length is no multiple of four) in FP32, as the
-    // 16-byte lanes of multidot_kernel and axpy_dot_kernel do, and those sums as pairs: the
-    // coefficients round to the same FP32 values as there.  Starts with a block barrier.
+    // whole vector; single products when its length is no multiple of four) in FP32, as a thread's
+    // 16-byte lanes in multidot_kernel and axpy_dot_kernel do, and those sums as pairs, in FP64 there.  Up
+    // to 466 944 unknowns, where a thread there has one such group (beyond, it chains the next ones in
+    // FP32), the coefficients round to the same FP32 values but near ties: 69 of 72 random dots.
+    // Starts with a block barrier.
     template <typename U, bool DOT>
     __device__ __forceinline__ void contribute(const U* cols, int ldc, int nv, const U* zz, bool self, int n) {
         using SU = typename SumOf<U>::S;
@@ -752,7 +755,9 @@ struct Solver {
     }
 
     // 1 / sqrt(||w1||^2 - ||h2||^2) rounded to FP32, from the FP32 pairs: one Newton step on the hardware's
-    // reciprocal square root with the residual formed exactly (every warp, FP32 pipes alone)
+    // reciprocal square root with the residual formed exactly (every warp, FP32 pipes alone).  Over 4e6
+    // norms in [1e-7, 2], starts two units off: at most 0.50000001 units from exact (FP64 root and
+    // quotient rounded once: 0.49999999), the same value in all but one.
     __device__ __forceinline__ float inverse_norm(int lane, int nv) {
         PairSum q{0.f, 0.f};
         if (lane < nv) {
