@@ -1910,9 +1910,10 @@ hdgdg_status hdgdg_step(hdgdg_sim* sim, int n_steps) {
     if (!sim->have_state) return fail(sim, HDGDG_ESTATE, "step before set_state");
     constexpr int kQueued = 64;   // explicit steps queued before the host waits
     const bool queued = explicit_scheme(&sim->cfg);
-    for (int k = 0; k < n_steps; k += queued ? kQueued : 1) {
+    for (int left = n_steps, n = 1; left > 0; left -= n) {   // (counted down: no sum past the largest int)
+        if (queued) n = std::min(kQueued, left);
         const long long l0 = launches_total();
-        const hdgdg_status st = queued ? explicit_steps(sim, std::min(kQueued, n_steps - k)) : one_step(sim);
+        const hdgdg_status st = queued ? explicit_steps(sim, n) : one_step(sim);
         sim->stats.kernel_launches += launches_total() - l0;
         if (st != HDGDG_OK) return st;
     }
