@@ -368,13 +368,12 @@ hdgdg_status hdgdg_stage_solve(hdgdg_sim* sim, const double* R1, double* Q, doub
  * solves are not one launch. */
 hdgdg_status hdgdg_set_solve_blocks(hdgdg_sim* sim, int blocks);
 
-/* Failure detection of the trace solves that run as one launch (host_steps): its blocks wait for one
- * another, each wait for at most `loads` loads (0 = the default, 2^22 trips to the L2 cache, a few
- * seconds); where one runs out the launch ends and the step or stage solve returns ECUDA, the state
- * left at the last completed step, from which the handle can go on.  lost = 1
- * (tests): one contribution to the next exchange is taken back, so that its waits run out.  EINVAL
+/* Failure detection of the trace solves that run as one launch (host_steps), for tests: one
+ * contribution to the next exchange between the launch's blocks is taken back, so that their waits run
+ * out (each is bounded, to about a second).  The launch then ends and the step or stage solve
+ * returns ECUDA, the state left at the last completed step, from which the handle can go on.  EINVAL
  * for a handle whose solves are not one launch. */
-hdgdg_status hdgdg_set_solve_wait(hdgdg_sim* sim, unsigned loads, int lost);
+hdgdg_status hdgdg_lose_contribution(hdgdg_sim* sim);
 
 /* ---- measurement helpers --------------------------------------------------------- */
 

@@ -371,7 +371,6 @@ struct hdgdg_sim {
     SolvePlan splan, splan_create;     // as it runs now, and as laid out at create (one block an SM)
     unsigned long long* solve_part = nullptr;
     unsigned* solve_epoch = nullptr;   // then the count, and at 16 words the launch's SolveClocks
-    unsigned solve_spins = kSolveMaxSpins;   // bound of its waits
     std::vector<StepGraph> step_graphs;   // whole-step graphs (host_steps = 0, timers off)
     SolveCtl* sctl = nullptr;             // device-side control of the solve being replayed
     DevHist* dhist = nullptr;             // each stage's guess history, as the step graph reads it
@@ -975,7 +974,6 @@ cudaError_t solve_enqueue_one_launch(hdgdg_sim* sim, const double* g, double* qh
     a.epoch = sim->solve_epoch;
     a.count = sim->solve_epoch + 1;
     a.error = spmv_error(sim);
-    a.max_spins = sim->solve_spins;
     a.dh = dh;
     std::memcpy(a.coef, kGuessCoef, sizeof(kGuessCoef));
     a.rtol = sim->cfg.krylov_rtol > 0.0 ? sim->cfg.krylov_rtol : (kMixed ? 1e-9 : 1e-15);
@@ -2159,19 +2157,15 @@ hdgdg_status hdgdg_set_solve_blocks(hdgdg_sim* sim, int blocks) {
     return HDGDG_OK;
 }
 
-hdgdg_status hdgdg_set_solve_wait(hdgdg_sim* sim, unsigned loads, int lost) {
+hdgdg_status hdgdg_lose_contribution(hdgdg_sim* sim) {
     if (!sim) return HDGDG_EINVAL;
     if (!sim->splan.on) return fail(sim, HDGDG_EINVAL, "this handle's trace solves are not one launch");
-    sim->solve_spins = loads > 0 ? loads : kSolveMaxSpins;
-    drop_step_graphs(sim);   // (the bound is an argument of the captured launch)
-    if (lost) {
-        unsigned count = 0;
-        CU(cudaMemcpyAsync(&count, sim->solve_epoch + 1, sizeof(count), cudaMemcpyDeviceToHost, sim->stream));
-        CU(cudaStreamSynchronize(sim->stream));
-        count -= 1u;
-        CU(cudaMemcpyAsync(sim->solve_epoch + 1, &count, sizeof(count), cudaMemcpyHostToDevice, sim->stream));
-        CU(cudaStreamSynchronize(sim->stream));
-    }
+    unsigned count = 0;
+    CU(cudaMemcpyAsync(&count, sim->solve_epoch + 1, sizeof(count), cudaMemcpyDeviceToHost, sim->stream));
+    CU(cudaStreamSynchronize(sim->stream));
+    count -= 1u;
+    CU(cudaMemcpyAsync(sim->solve_epoch + 1, &count, sizeof(count), cudaMemcpyHostToDevice, sim->stream));
+    CU(cudaStreamSynchronize(sim->stream));
     return HDGDG_OK;
 }
 

@@ -44,6 +44,7 @@ namespace {
 constexpr int kNT = kSolveThreads, kNW = kNT / 32;
 constexpr int kCtlWarps = 2;                    // warps 0 and 1: Hessenberg column, rotation, stop test
 constexpr int kProdThreads = kNT - 32 * kCtlWarps;
+constexpr unsigned kMaxSpins = 1u << 22;        // bound of every wait: loads, each a trip to L2 (0.8 s)
 
 // Values that cross blocks: each 32-bit half in an 8-byte word (accessed at once) under the 32-bit
 // number of the exchange it belongs to.
@@ -181,20 +182,16 @@ struct Solver {
     }
 
     // Whether to stop waiting after `spins` fruitless loads: the error word is then set, and every later
-    // wait of every block ends early.
+    // wait of every block ends early.  (A bound that is no constant -- an argument of the launch, a word in
+    // memory -- took 0.5 to 1 % of 8^2, k = 2, FP64.)
     __device__ __forceinline__ bool give_up(unsigned spins) {
         if ((spins & 63u) != 63u) return false;
-        if (*(volatile int*)&sh.gave_up == 0 && *reinterpret_cast<volatile int*>(a.error) == 0 && spins < a.max_spins)
+        if (*(volatile int*)&sh.gave_up == 0 && *reinterpret_cast<volatile int*>(a.error) == 0 && spins < kMaxSpins)
             return false;
         atomicExch(a.error, 3);
         *(volatile int*)&sh.gave_up = 1;
         return true;
     }
-
-    // A block barrier, and whether a wait of this block has run out: one answer for every thread.  (Read
-    // after the barrier, the flag may already be set by a thread that has gone on to its next wait; the
-    // threads that saw it would leave, and the others wait for them at a barrier without end.)
-    __device__ __forceinline__ bool any_gave_up() { return __syncthreads_or(*(volatile int*)&sh.gave_up) != 0; }
 
     __device__ __forceinline__ u64* a_buffer() {
         return a.A + (size_t)abuf * a.n_edges * NF * Tagged<T>::kWords;
@@ -273,7 +270,9 @@ struct Solver {
     // the partials themselves costs more the more blocks poll them (152 blocks, 6 columns: 8600
     // cycles an exchange, and 6600 through one owner a column; a counter and its poll 2500) -- and
     // the partials are then read once; their tags, not the count, say that they are there.
-    // Ends with a block barrier; false when a wait ran out.
+    // Ends with a block barrier and reads the flag of a wait that ran out (false: leave).  Every thread has
+    // to read the same, so the caller's next wait comes after another block barrier: a thread that went on
+    // into it could set the flag, those that saw it would leave and the others wait for them without end.
     template <typename U>
     __device__ __forceinline__ bool collect(int ncols, double* out, T* outt = nullptr, PairSum* outp = nullptr) {
         using SU = typename SumOf<U>::S;
@@ -319,7 +318,8 @@ struct Solver {
                 if (outp) outp[c] = s;
             }
         }
-        return !any_gave_up();
+        __syncthreads();
+        return sh.gave_up == 0;
     }
 
     // The neighbour traces of ng own edge rows from g0 on, of the vector published in `buf` by the
@@ -795,9 +795,9 @@ struct Solver {
             const int tid = thread_index();
             if (tid >= 32 * kCtlWarps) product(tid - 32 * kCtlWarps, a_buffer(), tag, V + j * ld);
             else if (j > 0) control(j - 1);
-            const bool out = any_gave_up();
+            __syncthreads();
             mark(0);
-            if (out) return -1;
+            if (sh.gave_up) return -1;   // (the next wait follows contribute's barriers)
             if (j > 0 && sh.done) return j;
             contribute<T, true>(V, ld, j + 1, z, false, R);
             if (!collect<T>(j + 1, sh.h1, h1t)) return -1;
@@ -841,9 +841,9 @@ struct Solver {
             const int tid = thread_index();
             if (tid >= 32 * kCtlWarps) product(tid - 32 * kCtlWarps, a_buffer(), tag, ao);
             else if (j > 0) control(j - 1);
-            const bool out = any_gave_up();
+            __syncthreads();
             mark(0);
-            if (out) return -1;
+            if (sh.gave_up) return -1;   // (the next wait follows contribute's barriers)
             if (j > 0 && sh.done) return j;
             if (j == 0) {
                 for (int r = tid; r < R; r += kNT) {
@@ -877,7 +877,9 @@ struct Solver {
             tag = epoch;
             abuf ^= 1u;
             first_pass(tid, j + 1, ao, true);
-            if (!second_dots(j + 1, ao)) return -1;
+            const bool there = second_dots(j + 1, ao);
+            __syncthreads();   // (the next product waits without another barrier: see collect)
+            if (!there) return -1;
             mark(1);
             if (j == a.m - 1) {
                 if (tid < 32 * kCtlWarps) control(j);

@@ -9,7 +9,6 @@ namespace hdgdg {
 
 constexpr int kSolveThreads = 512;
 constexpr int kSolveMaxBlocks = 256;
-constexpr unsigned kSolveMaxSpins = 1u << 22;     // default bound of a wait: loads, each a trip to L2 (seconds)
 constexpr int kSolveMaxCols = GmresCtl::kM + 1;   // columns of one reduction: 32 basis vectors and a norm
 
 // How a handle's system is laid out over the launch's blocks (plan_solve, fixed at create).
@@ -59,7 +58,6 @@ struct SolveArgs {
     unsigned* epoch;             // the last exchange's number, kept between launches
     unsigned* count;             // contributions to exchanges (epoch x blocks, modulo 2^32)
     int* error;                  // set when a bounded wait ran out
-    unsigned max_spins;          // bound of every wait, in loads
     const DevHist* dh;           // guess history (nullptr: none)
     bool start_given;            // x~ = xt, w and sc are already set (the least-squares start)
     double coef[7][6];

@@ -22,7 +22,7 @@ DG_PRECISIONS = {"default": 0, "bf16": 1}
 EXPORTS = ["hdgdg_bytes_required", "hdgdg_node_coords", "hdgdg_create", "hdgdg_set_state",
            "hdgdg_step", "hdgdg_get_state", "hdgdg_get_stats", "hdgdg_last_error", "hdgdg_destroy",
            "hdgdg_update_state", "hdgdg_eval_nl", "hdgdg_condense_rhs", "hdgdg_trace_apply", "hdgdg_set_trace_tile", "hdgdg_set_local_tiles",
-           "hdgdg_stage_solve", "hdgdg_set_solve_blocks", "hdgdg_set_solve_wait",
+           "hdgdg_stage_solve", "hdgdg_set_solve_blocks", "hdgdg_lose_contribution",
            "hdgdg_measure_fp64_tflops", "hdgdg_measure_conversion_rates", "hdgdg_set_kernel_timing", "hdgdg_kernel_time",
            "hdgdg_mass_noalloc", "hdgdg_gll", "hdgdg_checkpoint_bytes", "hdgdg_save_checkpoint",
            "hdgdg_load_checkpoint", "hdgdg_ensemble_create", "hdgdg_ensemble_set_state", "hdgdg_ensemble_step",
@@ -96,7 +96,7 @@ def lib():
         L.hdgdg_set_trace_tile.argtypes = [ctypes.c_void_p, ctypes.c_int]
         L.hdgdg_set_local_tiles.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
         L.hdgdg_set_solve_blocks.argtypes = [ctypes.c_void_p, ctypes.c_int]
-        L.hdgdg_set_solve_wait.argtypes = [ctypes.c_void_p, ctypes.c_uint, ctypes.c_int]
+        L.hdgdg_lose_contribution.argtypes = [ctypes.c_void_p]
         L.hdgdg_stage_solve.argtypes = [ctypes.c_void_p, _P, _P, _P, ctypes.POINTER(ctypes.c_int)]
         L.hdgdg_measure_fp64_tflops.argtypes = [_P]
         L.hdgdg_measure_conversion_rates.argtypes = [_P, _P]
@@ -355,9 +355,9 @@ class Sim:
         """Blocks of the one-launch trace solves: < 0 one an SM, 0 a launch per operation, n at most n."""
         self._check(lib().hdgdg_set_solve_blocks(self._h, int(blocks)))
 
-    def set_solve_wait(self, loads=0, lost=False):
-        """Bound the waits of the one-launch trace solves (0: the default); lost: let the next one run out."""
-        self._check(lib().hdgdg_set_solve_wait(self._h, int(loads), int(bool(lost))))
+    def lose_contribution(self):
+        """Tests: the next one-launch trace solve's waits run out (HdgdgError ECUDA)."""
+        self._check(lib().hdgdg_lose_contribution(self._h))
 
     def stage_solve(self, R1):
         R1 = _f64(R1, (3, self.n_el, self.Np))
