@@ -1017,8 +1017,7 @@ hdgdg_status solve_one_launch(hdgdg_sim* sim, const double* g, double* qhat, int
     StepStats ss;
     std::memcpy(flag, sim->hbuf, sizeof(flag));
     std::memcpy(&ss, sim->hbuf + 4, sizeof(ss));
-    if (flag[3]) return solve_wait_ran_out(sim, flag[3]);
-    if (eb) {   // the launch's time, divided among the kernel classes as its first block's clock saw them
+    if (eb && !flag[3]) {   // the launch's time, divided among the kernel classes as its first block's clock saw them
         SolveClocks ck;
         std::memcpy(&ck, sim->hbuf + 16, sizeof(ck));
         const long long part[5] = {ck.spmv, ck.ortho, ck.residual, ck.guess, ck.precond};
@@ -1038,6 +1037,7 @@ hdgdg_status solve_one_launch(hdgdg_sim* sim, const double* g, double* qhat, int
     }
     if (ea) sim->ev_pool.push_back(ea);
     if (eb) sim->ev_pool.push_back(eb);
+    if (flag[3]) return solve_wait_ran_out(sim, flag[3]);
     *iters = ss.last_its;
     *relres = ss.last_rel;
     sim->stats.last_krylov_iterations = ss.last_its;

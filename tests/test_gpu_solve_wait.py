@@ -74,3 +74,21 @@ def test_the_handle_goes_on_after_a_lost_contribution(form, host_steps):
         with pytest.raises(hd.HdgdgError):
             s.stage_solve(R1)
         assert np.array_equal(s.stage_solve(R1)[1], want)
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_the_timers_leave_a_failed_launch_out(form):
+    """With the kernel-class timers on, the launch that gave up after most of a second is in no class, and
+    the steps after it are timed."""
+    h, hu, hv, b, dt = _state(24, 3)
+    with hd.Sim(24, 3, dt, bottom=b, **FORMS[form]) as s:
+        s.set_state(h, hu, hv)
+        s.set_kernel_timing(True)
+        s.step(2)
+        s.lose_contribution()
+        with pytest.raises(hd.HdgdgError):
+            s.step(1)
+        s.step(2)
+        times = s.kernel_times()
+    assert all(times[c][0] > 0.0 for c in ("spmv", "ortho", "residual", "guess", "precond"))
+    assert sum(ms for ms, _ in times.values()) < 100.0
